@@ -99,9 +99,10 @@ int cg_context_destroy(cg_context *ctx);
 /*
  * LexBFS order of a dense graph (Section 4.2: pick the first vertex of the
  * first class, split every class C into C ∩ N_x placed before C \ N_x;
- * Section 6.1 runs it on the GPU).  One persistent CTA walks all n steps with
- * the partition state in shared memory (n <= 16384), split between shared
- * memory and the workspace (n <= 65520) or in the workspace.
+ * Section 6.1 runs it on the GPU).  One persistent CTA numbers up to 32
+ * vertices per pass over the partition, whose state is in shared memory
+ * (n <= 19904), split between shared memory and the workspace (n <= 42624) or
+ * mostly in the workspace.
  *   g      device graph, n >= 0, n <= 131072
  *   order  device int32[n] (written)
  *   pos    device int32[n] (written) or NULL

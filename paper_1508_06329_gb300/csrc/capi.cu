@@ -27,14 +27,11 @@ int set_error(int status, const char *fmt, ...) {
 const char *cg_debug_array_name(unsigned code) {
     switch (code) {
         case kChkCls: return "dense LexBFS cls";
-        case kChkChild: return "dense LexBFS child";
-        case kChkFree: return "dense LexBFS free stack";
-        case kChkCnext: return "dense LexBFS class next";
-        case kChkCprev: return "dense LexBFS class prev";
-        case kChkSize: return "dense LexBFS class size";
+        case kChkPerm: return "dense LexBFS positions";
+        case kChkKey: return "dense LexBFS keys";
+        case kChkSplit: return "dense LexBFS split words";
+        case kChkSort: return "dense LexBFS split sort";
         case kChkNumbered: return "dense LexBFS numbered mask";
-        case kChkRow: return "dense LexBFS pivot row";
-        case kChkMoved: return "dense LexBFS moved counts";
         case kChkCsrCls: return "CSR LexBFS cls";
         case kChkCsrVnext: return "CSR LexBFS vnext";
         case kChkCsrVprev: return "CSR LexBFS vprev";
@@ -243,16 +240,6 @@ int make_layout(cg_context *ctx, const cg_dense *graphs, int32_t count, const in
         const int cnt = B.end - B.begin;
         if (b < 9) {
             if ((rc = fused_dense_plan(B.nmax, ctx->tuned_threads[b], &B.fplan))) return rc;
-            if (B.fplan.rows_smem) {
-                // rows in shared memory make a step faster but can leave one CTA per SM;
-                // with more graphs than that wave holds, rows read from L2 (a step
-                // ~1.3x slower) and more CTAs per SM take fewer waves
-                FusedPlan pg;
-                if ((rc = fused_dense_plan(B.nmax, ctx->tuned_threads[b], &pg, false))) return rc;
-                const int64_t ws = ceil_div(cnt, (int64_t)ctx->num_sms * fused_ctas_per_sm(B.fplan));
-                const int64_t wg = ceil_div(cnt, (int64_t)ctx->num_sms * fused_ctas_per_sm(pg));
-                if (wg * 13 < ws * 10) B.fplan = pg;
-            }
             B.ctas = std::min(cnt, ctx->num_sms * fused_ctas_per_sm(B.fplan));
         } else {
             if ((rc = lexbfs_dense_plan(B.nmax, ctx->cfg.threads_override, &B.lplan))) return rc;
@@ -281,7 +268,6 @@ BatchBuffers batch_buffers(const BatchLayout &L, bool need_order) {
     bb.o_voff = cv.take<int64_t>(L.count + 1);
     bb.o_order = cv.take<int32_t>(need_order ? L.total : 0);
     bb.o_pos = cv.take<int32_t>(L.total);
-    bb.o_parent = cv.take<int32_t>(L.total);
     bb.o_ppos = cv.take<int32_t>(L.total);
     // + the check's CTA counter and error word (bucket 9 is last)
     bb.o_keys = cv.take<unsigned long long>(L.count + 2);
@@ -304,7 +290,7 @@ int enqueue_batch(cg_context *ctx, const BatchLayout &L, const BatchBuffers &bb,
     const DenseDesc *ddesc = reinterpret_cast<const DenseDesc *>(P(bb.o_desc));
     int32_t *order = orders ? orders : reinterpret_cast<int32_t *>(P(bb.o_order));
     int32_t *pos = reinterpret_cast<int32_t *>(P(bb.o_pos));
-    int32_t *parent = reinterpret_cast<int32_t *>(P(bb.o_parent));
+    int32_t *ppos = reinterpret_cast<int32_t *>(P(bb.o_ppos));
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(P(bb.o_keys));
     int *counters = reinterpret_cast<int *>(P(bb.o_counter));
     CG_CUDA_TRY(cudaEventRecord(ss.fork, stream));
@@ -317,18 +303,17 @@ int enqueue_batch(cg_context *ctx, const BatchLayout &L, const BatchBuffers &bb,
         CG_CUDA_TRY(cudaStreamWaitEvent(s, ss.fork, 0));
         if (b < 9) {
             PhaseTimer pt(tctx, &ctx->ev_fused, s);
-            if ((rc = fused_dense_launch(B.fplan, ddesc + B.begin, cnt, B.ctas, order, pos, parent, res,
-                                         counters + 64 * b, s)))
+            if ((rc = fused_dense_launch(B.fplan, ddesc + B.begin, cnt, B.ctas, order, ppos, res, counters + 64 * b,
+                                         s)))
                 return rc;
             if (account) ctx->launches += 1;
         } else {
-            int32_t *ppos = reinterpret_cast<int32_t *>(P(bb.o_ppos));
             uint32_t *emask = B.stage ? reinterpret_cast<uint32_t *>(P(bb.o_emask)) : nullptr;
             {
                 PhaseTimer pt(tctx, &ctx->ev_lex, s);
                 if ((rc = lexbfs_dense_launch(B.lplan, ddesc + B.begin, DenseDesc{}, cnt, B.ctas, order, pos, ppos,
                                               B.lplan.gstate_bytes ? P(bb.o_gstate) : nullptr, counters + 64 * b, s,
-                                              kParentPivots, keys + B.begin, emask, parent)))
+                                              keys + B.begin, emask)))
                     return rc;
             }
             PhaseTimer pt(tctx, &ctx->ev_check, s);
@@ -377,12 +362,11 @@ int upload_layout(cg_context *ctx, const BatchLayout &L, const BatchBuffers &bb,
 
 // Workspace layout of run_single_dense (also the start of the host entry's).
 struct SingleDenseCarve {
-    size_t o_order, o_pos, o_parent, o_ppos, o_key, o_counter, o_gstate, o_emask;
+    size_t o_order, o_pos, o_ppos, o_key, o_counter, o_gstate, o_emask;
     Carve cv;
     SingleDenseCarve(int n, const LexPlan &plan) {
         o_order = cv.take<int32_t>(n);
         o_pos = cv.take<int32_t>(n);
-        o_parent = cv.take<int32_t>(n);
         o_ppos = cv.take<int32_t>(n);
         o_key = cv.take<unsigned long long>(3);   // key, the check's CTA counter, error word
         o_counter = cv.take<int>(1);
@@ -405,26 +389,25 @@ int run_single_dense(cg_context *ctx, const cg_dense *g, int32_t *order_out, int
     if ((rc = ensure_ws(ctx, base + sc.cv.off))) return rc;
     int32_t *order = order_out ? order_out : at<int32_t>(ctx, base + sc.o_order);
     int32_t *pos = pos_out ? pos_out : at<int32_t>(ctx, base + sc.o_pos);
-    int32_t *parent = at<int32_t>(ctx, base + sc.o_parent);
     unsigned long long *key = at<unsigned long long>(ctx, base + sc.o_key);
     const DenseDesc d = desc_of(g, 0, 0);
+    int32_t *ppos = at<int32_t>(ctx, base + sc.o_ppos);
     if (n == 0) {
         if (!res) return CG_OK;
         PhaseTimer pt(ctx, &ctx->ev_check, stream);
         ctx->launches += 1;
-        return peo_dense_launch(nullptr, d, 1, nullptr, 0, order, pos, parent, true, key, ctx->num_sms, stream,
+        return peo_dense_launch(nullptr, d, 1, nullptr, 0, order, pos, ppos, true, key, ctx->num_sms, stream,
                                 nullptr, 0, false, res);
     }
     // with a result wanted, the search also records the parents of its pivots
     // by position (one store per step) and initialises the check's keys
-    int32_t *ppos = at<int32_t>(ctx, base + sc.o_ppos);
     const bool stage = res && peo_stage_ok(d);
     uint32_t *emask = stage ? at<uint32_t>(ctx, base + sc.o_emask) : nullptr;
     {
         PhaseTimer pt(ctx, &ctx->ev_lex, stream);
         rc = lexbfs_dense_launch(plan, nullptr, d, 1, 1, order, pos, res ? ppos : nullptr,
-                                 plan.gstate_bytes ? at<void>(ctx, base + sc.o_gstate) : nullptr, at<int>(ctx, base + sc.o_counter),
-                                 stream, kParentPivots, res ? key : nullptr, emask, res ? parent : nullptr);
+                                 plan.gstate_bytes ? at<void>(ctx, base + sc.o_gstate) : nullptr,
+                                 at<int>(ctx, base + sc.o_counter), stream, res ? key : nullptr, emask);
         if (rc) return rc;
         ctx->launches += 1;
     }
@@ -1129,15 +1112,13 @@ int cg_batch_autotune(cg_context *ctx, const cg_dense *graphs, int32_t count, cu
             if ((rc = upload_layout(ctx, L, bb, base, stream))) break;
             const auto &B = L.bk[bk];
             int32_t *order = reinterpret_cast<int32_t *>(base + bb.o_order);
-            int32_t *pos = reinterpret_cast<int32_t *>(base + bb.o_pos);
-            int32_t *parent = reinterpret_cast<int32_t *>(base + bb.o_parent);
+            int32_t *ppos = reinterpret_cast<int32_t *>(base + bb.o_ppos);
             const DenseDesc *dd = reinterpret_cast<const DenseDesc *>(base + bb.o_desc);
             int *ctr = reinterpret_cast<int *>(base + bb.o_counter);
             float ms = 0.f;
             for (int rep = 0; rep < 2 && rc == CG_OK; ++rep) {   // second run is timed
                 cudaEventRecord(a, stream);
-                rc = fused_dense_launch(B.fplan, dd + B.begin, B.end - B.begin, B.ctas, order, pos, parent, res, ctr,
-                                        stream);
+                rc = fused_dense_launch(B.fplan, dd + B.begin, B.end - B.begin, B.ctas, order, ppos, res, ctr, stream);
                 cudaEventRecord(b, stream);
                 cudaEventSynchronize(b);
                 cudaEventElapsedTime(&ms, a, b);

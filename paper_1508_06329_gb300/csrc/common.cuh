@@ -138,7 +138,7 @@ __device__ __forceinline__ T *cg_arr(T *p, unsigned long long, unsigned) {
 
 // Array codes of the bounds-checking build (the high byte of the error word).
 enum : unsigned {
-    kChkCls = 1, kChkChild, kChkFree, kChkCnext, kChkCprev, kChkSize, kChkNumbered, kChkRow, kChkMoved,
+    kChkCls = 1, kChkPerm, kChkKey, kChkSplit, kChkSort, kChkNumbered,
     kChkCsrCls = 16, kChkCsrVnext, kChkCsrVprev, kChkCsrCnext, kChkCsrCprev, kChkCsrCfirst, kChkCsrClast,
     kChkCsrCsize, kChkCsrCmoved, kChkCsrCchild, kChkCsrFree, kChkCsrSy, kChkCsrSop, kChkCsrSon, kChkCsrSrun,
     kChkCsrSkey,
@@ -148,10 +148,6 @@ enum : unsigned {
 
 // Parent value meaning "not known yet": the dense check finds it.
 constexpr int kParentUnresolved = -2;
-
-// How the dense LexBFS records parents (when given a parent array).
-constexpr int kParentMoves = 0;        // every moved vertex: parent[v] = pivot
-constexpr int kParentPivots = 1;       // once per step, by position: parent[i], or kParentUnresolved
 
 // Per-graph descriptor as the kernels see it (device memory).
 struct DenseDesc {

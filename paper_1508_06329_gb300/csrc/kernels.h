@@ -11,12 +11,10 @@ namespace cg {
 // ---- dense LexBFS (lexbfs_dense.cu)
 struct LexPlan {
     int threads;        // CTA size
-    bool rows_smem;     // adjacency copied into shared memory
-    bool wide_ids;      // 32-bit ids, state in a global workspace
-    int split_state;    // 16-bit ids, class ids in shared memory, class arrays partly in a global
-                        // workspace: 0 no, else the split layout 2, 3 or 5 (lexbfs_dense.cuh)
+    int state;          // where the per-vertex arrays live (kState* of lexbfs_dense.cuh)
+    int sort_cap;       // elements of the split sort's arrays
     size_t smem_bytes;  // dynamic shared memory per CTA
-    size_t gstate_bytes;// global state bytes per CTA (0: none)
+    size_t gstate_bytes;// workspace bytes per CTA (0: none)
     int n_max;          // the largest graph the plan was made for
 };
 
@@ -27,21 +25,16 @@ int lexbfs_dense_plan(int n_max, int threads_override, LexPlan *plan);
 // Runs LexBFS for `count` graphs, one CTA each (grid = min(count, ctas)).
 // descs: device array, or nullptr to use `single` (count must be 1).
 // work_counter: device int, zeroed by the launcher (dynamic graph hand-out).
-// parent (packed by vbase) receives parents when non-null: parent_mode
-// kParentMoves records p(v) for every vertex (a store per moved vertex),
-// kParentPivots one value per step by position, parent[i] = p(order[i]), or
-// kParentUnresolved for the pivots chosen by a class scan.  keys (nullable)
+// ppos (nullable, packed by vbase) receives the parents by position:
+// ppos[i] = p(order[i]), -1 when it has no earlier neighbour.  keys (nullable)
 // is set, on the stream after the search, to the check's initial keys:
 // keys[0..count) = "no violation", keys[count] = keys[count + 1] = 0.
 // emask (nullable): the search also writes each graph's earlier-than masks
 // E_b (b >= 1; row b at emask + ebase + b * mask_stride(n): the vertices
-// numbered before step 32 b), which the staged check reads.  cpar
-// (nullable; n ints per graph at vbase, scratch) makes kParentPivots exact:
-// no kParentUnresolved is left.
+// numbered before step 32 b), which the staged check reads.
 int lexbfs_dense_launch(const LexPlan &plan, const DenseDesc *descs, DenseDesc single, int count, int ctas,
-                        int32_t *order, int32_t *pos, int32_t *parent, void *gstate, int *work_counter,
-                        cudaStream_t stream, int parent_mode = 0, unsigned long long *keys = nullptr,
-                        uint32_t *emask = nullptr, int32_t *cpar = nullptr);
+                        int32_t *order, int32_t *pos, int32_t *ppos, void *gstate, int *work_counter,
+                        cudaStream_t stream, unsigned long long *keys = nullptr, uint32_t *emask = nullptr);
 
 // Bounds-checking build: the next dense LexBFS launch records `code` (a test
 // of the error path); CG_EINVAL in the release build.
@@ -99,17 +92,15 @@ int finalize_launch(const DenseDesc *descs, DenseDesc single, int count, const u
 
 // ---- fused small-graph test, one CTA per graph (batch_dense.cu)
 constexpr int kFusedMaxN = 4096;
-constexpr size_t kFusedSmemLimit = 227 * 1024 - 64;
 struct FusedPlan {
     int threads;
-    bool rows_smem;
+    int sort_cap;
     size_t smem_bytes;
 };
-// threads = 0 picks by size; otherwise 64, 128, 256 or 512.  The rows are
-// copied to shared memory when they fit and rows_smem_allowed.
-int fused_dense_plan(int n_max, int threads, FusedPlan *plan, bool rows_smem_allowed = true);
+// threads = 0 picks by size; otherwise 64, 128, 256 or 512.
+int fused_dense_plan(int n_max, int threads, FusedPlan *plan);
 int fused_dense_launch(const FusedPlan &plan, const DenseDesc *descs, int count, int ctas, int32_t *order,
-                       int32_t *pos, int32_t *parent, cg_result *res, int *work_counter, cudaStream_t stream);
+                       int32_t *ppos, cg_result *res, int *work_counter, cudaStream_t stream);
 int fused_ctas_per_sm(const FusedPlan &plan);
 
 // ---- one multi-sweep LexBFS sweep on a dense graph (sweep_dense.cu)

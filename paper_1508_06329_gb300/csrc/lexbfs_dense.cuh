@@ -1,523 +1,786 @@
-// lexbfs_dense.cuh — LexBFS by partition refinement, one CTA per graph.
+// lexbfs_dense.cuh — LexBFS by partition refinement in panels of up to 32
+// pivots, one CTA per graph.
 //
 // Method (Section 4.2 of the paper; its GPU form in Section 6.1): the
 // unnumbered vertices are partitioned into classes ordered top first.  Each
-// step visits the first vertex x of the first class, then replaces every
-// class C by C ∩ N_x followed by C \ N_x (Observation 6.2: the new class goes
-// right before the class it came from).  Within a class vertices are kept in
-// id order, so the visited vertex is the lowest id of the top class.
+// step visits the first vertex x of the first class, then replaces every class
+// C by C ∩ N_x followed by C \ N_x.  Within a class vertices are kept in id
+// order, so the visited vertex is the lowest id of the top class.
 //
-// GPU form used here (differs from the paper's four kernels per step, whose
-// racy pick and racy set creation are replaced by deterministic rules):
-//   * state: cls[v] (class id per vertex), a doubly linked class list with a
-//     head sentinel, and per class one word packing (size, moved-this-step);
-//     everything sits in shared memory for n <= 16384 (16-bit ids), otherwise
-//     in a global workspace (32-bit ids);
-//   * the pivot row is read word-parallel (thread t owns words t, t+T, ...);
-//     each unnumbered neighbour y bumps the moved count of its class with a
-//     shared-memory atomic; the first arrival per class is its allocator;
-//   * allocators split a class only when it loses some but not all members
-//     (C ∩ N_x and C \ N_x both non-empty), taking a fresh id from a free
-//     stack and linking it right before C;  a class that moves entirely keeps
-//     its id and place;
-//   * the relabel cls[y] = child[cls[y]] of a step's moved vertices is
-//     deferred to the next step and done by the thread owning y's word;
-//   * the next pivot is the lowest moved vertex of the top class (an atomicMin
-//     collected while splitting), or of the class after it when the top class
-//     empties; only when neither class lost members is a class scan needed.
-//     A known pivot's row is requested right after the first barrier, so its
-//     load overlaps the list update, the second barrier and the next step's
-//     relabel pass.  Two __syncthreads per step;
-//   * a shared bitmask of numbered vertices filters each pivot row, so only
-//     unnumbered neighbours are visited; the deferred relabel and the split
-//     are two short loops over a word's bits, and a thread posts only its
-//     first (lowest) candidate of the top class to the pivot atomicMin;
-//   * parents: p(y) of the perfect-elimination check (Section 5.2), y's
-//     neighbour with the largest order index below its own, is the last pivot
-//     that moved y.  kParentMoves stores it for every moved vertex (one store
-//     per edge; the one-CTA fused test wants all parents).  kParentPivots
-//     stores one value per step, by position (parent[i] = p(order[i])): a
-//     pivot chosen among the moved vertices has the current pivot as parent;
-//     one chosen by a class scan gets kParentUnresolved and the check finds
-//     it, unless cpar is given: the members of a class share one label and
-//     so one latest numbered neighbour, the pivot that last moved them,
-//     which cpar[c] records (set by the allocators when a class is split off
-//     or moves whole).  A pivot scanned from the top class f shares the
-//     current pivot's parent; one scanned from the class after it reads
-//     cpar there (loaded by thread 0 at the start of the step);
-//   * with emask, the numbered bitmask at the start of every step 32 b
-//     (b >= 1) is also written out as E_b, the vertices numbered before
-//     position 32 b: the staged check reads one mask row per 32 positions
-//     instead of building it from pos;
-//   * the graph's rows are bulk-prefetched into L2 when the CTA starts.
+// One step at a time costs a row load, two CTA barriers and a pass over the
+// row per vertex (1.74 us per step at n = 16,384 on GB300, all of it latency
+// and issue).  But the steps of the classes in front do not need the rest of
+// the partition: every member of a class is visited before any member of a
+// later class, and the order of the members of the first classes depends only
+// on the edges among them.  So a panel takes the next (at most) 32 vertices in
+// partition order, the window:
+//   1. the threads read the window's rows, a word of all 32 rows per thread,
+//      and transpose the 32 x 32 bits in registers: vertex y's key, bit j =
+//      adjacent to window vertex j;
+//   2. the window vertices' own keys are the window's adjacency: every warp
+//      finds how many of them are visited in window order, in one comparison
+//      per lane (panel_in_order).  That is nearly always all of them; when it
+//      is fewer than kPanelFew, warp 0 runs LexBFS on the window, one lane per
+//      vertex (panel_solve);
+//   3. the classes whose members' keys differ are split: members in decreasing
+//      order of the key read in pivot order (the lexicographic order of the
+//      labels these r steps append), ids ascending among equals.
+// A window's last class may continue beyond it.  Then a pivot from its part in
+// the window is only taken while no member outside can have a larger label:
+// while its appended label is all ones, or, when that gives few pivots (large
+// independent sets), at least the OR of the outside members' keys; members
+// outside have larger ids, so equality suffices.  A panel numbers 26..32
+// vertices on chordal, dense random, sparse random and tree inputs.
+//
+// Measured on GB300 (whole test, before -> now): the pair of n = 16,384 graphs
+// at density 0.1 28.5 -> 4.7 ms (8.8 us per panel of 31), G(10,000, 0.5)
+// 49.7 -> 2.5 ms, n = 41,003 104.7 -> 33.5 ms, 4,096 graphs of 16..2,048
+// vertices 3.77 -> 1.53 ms, one graph of 1,000 vertices 919 -> 244 us.  What
+// bounds a panel is latency: the rows' L2 loads, the transpose's issue slots
+// and three CTA barriers.
+//
+// State: perm[] holds the vertices by position (numbered ones in front, then
+// class after class, ascending ids inside a class), and the class boundaries
+// are a bitmask over positions.  A class that does not split is not touched,
+// so a panel without splits costs steps 1, 2 and one pass over the positions
+// that compares neighbouring keys.  Splits: members with key 0 keep their
+// order and move to the end of the class (prefix counts), the others are
+// sorted by (class, key, order), by counting when the classes' moved parts are
+// small, else with a bitonic network.  More than cap of them (the first steps
+// on a dense random graph): the panel is cut to its first pivot, whose one-bit
+// keys need no sort.
+//
+// Parents: p(y) of the perfect-elimination check (Section 5.2), y's neighbour
+// with the largest order index below its own, is the last pivot whose bit is
+// set in y's label.  Members of a class share their label, so while a class is
+// unnumbered ppos[its first position] holds that pivot (-1: none); a pivot's
+// own parent is the last adjacent pivot of its panel or else that value.
+// emask: E_b, the vertices numbered before position 32 b, one mask row per 32
+// positions for the staged check.
 #pragma once
 #include "common.cuh"
 
 namespace cg {
 
-template <typename Id>
-struct IdTraits;
-template <>
-struct IdTraits<uint16_t> {
-    using Sz = uint32_t;
-    static constexpr int kShift = 16;
-    static constexpr uint32_t kMask = 0xFFFFu;
-};
-template <>
-struct IdTraits<uint32_t> {
-    using Sz = unsigned long long;
-    static constexpr int kShift = 32;
-    static constexpr unsigned long long kMask = 0xFFFFFFFFull;
-};
-
-template <typename Id>
-struct LexState {
-    CG_ARR(typename IdTraits<Id>::Sz) sz;  // [n]     size | moved-this-step << kShift (size only with mvw)
-    CG_ARR(uint32_t) mvw;                  // [(n+1)/2] moved-this-step, two 16-bit counts per word (split layouts 2, 3)
-    CG_ARR(uint16_t) mvh;                  // [n]     the same counts as 16-bit entries (stores)
-    CG_ARR(uint32_t) arrived;              // [ceil(n/32)] class c's bit: a member moved this step (layout 5)
-    CG_ARR(Id) cls;                        // [n]     class of each vertex, kNumbered once visited
-    CG_ARR(Id) child;                      // [n]     class receiving a class's pivot neighbours
-    CG_ARR(Id) freel;                      // [n]     stack of unused class ids
-    CG_ARR(Id) cnext;                      // [n + 1] class list; index n is the head sentinel
-    CG_ARR(Id) cprev;                      // [n + 1]
-    CG_ARR(uint32_t) numbered;             // [ceil(n/32)] bit v set once v is visited
-};
-
-struct LexScalars {
-    int free_top;
-    int next_graph;
-    unsigned front_min[2];
-    unsigned second_min[2];
-    unsigned split[2];   // a class was split in the step of this parity (its moved vertices need a relabel)
-    unsigned red[32];
-};
-
 constexpr unsigned kNoVertex = 0xFFFFFFFFu;
 
-// How lexbfs_cta records parents (when given a parent array).
+// Where the per-vertex arrays live.  A vertex's key is gathered once per panel
+// in position order, so the keys stay in shared memory as long as they fit;
+// perm is only read in order, so it moves to the workspace first.
+constexpr int kStateSmem = 0;       // perm and keys in shared memory, 16-bit ids
+constexpr int kStatePermGlobal = 1; // perm in the workspace, keys in shared memory, 16-bit ids
+constexpr int kStateGlobal = 2;     // perm and keys in the workspace, 32-bit ids
 
-template <typename Id>
-__host__ __device__ inline size_t lex_state_bytes(int n) {
-    using Sz = typename IdTraits<Id>::Sz;
-    size_t b = (size_t)n * sizeof(Sz) + (size_t)n * sizeof(Id) * 3 + (size_t)(n + 1) * sizeof(Id) * 2;
+template <int STATE>
+struct PanelId { using type = uint16_t; };
+template <>
+struct PanelId<kStateGlobal> { using type = uint32_t; };
+
+struct PanelScalars {
+    int piv[32];            // the panel's pivots in order
+    int par[32];            // their parents
+    uint32_t bit[32];       // window vertex j's bit in pivot order (0: not a pivot)
+    uint32_t tab[8][16];    // nibble tables of the same permutation
+    int scan[3][32];
+    int r;                  // pivots of the panel
+    uint32_t pivmask;       // window vertices that are pivots
+    int ident;              // the pivots are window vertices 0..r-1 in order
+    int cend;               // end of the class that goes on beyond the window
+    uint32_t ub;            // OR of the keys of its members beyond the window
+    int set_start;          // position whose boundary bit the commit set (-1: none)
+    int any;                // some class has members with different keys
+    int nz_max;             // the most moved members in one split class
+    int next_graph;
+};
+constexpr size_t kPanelScalarBytes = (sizeof(PanelScalars) + 15) & ~size_t(15);
+
+constexpr int kPanelWordArrays = 9;
+constexpr int kPanelFew = 16;   // pivots below which a panel is worth extending by slower rules
+constexpr int kSortCapMax = 4096;
+
+// Elements the split sort holds: all of a small graph's vertices, fewer when
+// the state leaves less room (bytes: shared memory available for them).
+__host__ __device__ inline int panel_sort_cap(int n, size_t bytes) {
+    int cap = kSortCapMax;
+    while (cap > 64 && (cap / 2 >= n || (size_t)cap * 12 > bytes)) cap /= 2;
+    return cap;
+}
+
+// Shared bytes of a graph of n vertices without the sort's arrays.
+__host__ __device__ inline size_t panel_state_bytes(int n, int state) {
+    const size_t wn = (size_t)(n + 31) / 32;
+    size_t b = wn * 4 * kPanelWordArrays;
     b = (b + 15) & ~size_t(15);
-    b += (size_t)((n + 31) / 32) * sizeof(uint32_t);   // numbered bitmask
-    return (b + 15) & ~size_t(15);
-}
-
-template <typename Id>
-__device__ inline LexState<Id> lex_state_carve(unsigned char *base, int n) {
-    using Sz = typename IdTraits<Id>::Sz;
-    LexState<Id> s;
-    s.sz = cg_arr(reinterpret_cast<Sz *>(base), n, kChkSize);
-    Id *p = reinterpret_cast<Id *>(base + (size_t)n * sizeof(Sz));
-    s.cls = cg_arr(p, n, kChkCls);
-    s.child = cg_arr(p + n, n, kChkChild);
-    s.freel = cg_arr(p + 2 * (size_t)n, n, kChkFree);
-    s.cnext = cg_arr(p + 3 * (size_t)n, n + 1, kChkCnext);
-    s.cprev = cg_arr(p + 4 * (size_t)n + 1, n + 1, kChkCprev);
-    size_t b = (size_t)n * sizeof(Sz) + (size_t)n * sizeof(Id) * 3 + (size_t)(n + 1) * sizeof(Id) * 2;
-    s.numbered = cg_arr(reinterpret_cast<uint32_t *>(base + ((b + 15) & ~size_t(15))), (n + 31) / 32, kChkNumbered);
-    return s;
-}
-
-constexpr size_t kLexScalarBytes = (sizeof(LexScalars) + 15) & ~size_t(15);
-
-// Split layouts for graphs too large for the whole state in shared memory but
-// within 16-bit ids.  The per-vertex class ids and the numbered bitmask (read
-// and written for every moved vertex and by class scans) always stay in
-// shared memory; of the per-class state, what a moved vertex touches goes
-// there too as far as it fits, the rest (sizes, the free stack and the class
-// list, touched once per split class) to a global workspace:
-//   layout 3 (n <= 37,920): the moved counts (16 bits each, two per word for
-//     the shared atomics) and the children;
-//   layout 2 (n <= 56,312): the moved counts;
-//   layout 5 (n <= 65,520): one "arrived" bit per class (the first moved
-//     member's atomicOr elects the class's allocator); the counts are added
-//     to the packed global size words without a return value.
-// (Arrival bits with the children in shared memory and the counts in global
-// memory, measured on GB300 for 37,921..54,656 vertices, matched layout 2 on
-// a sparse graph but were ~1.4x slower per step on a dense one, whose moved
-// vertices pile onto few global count words.)
-constexpr int kLayoutSplitMv = 2, kLayoutSplitMvChild = 3, kLayoutSplitArr = 5;
-__host__ __device__ constexpr bool layout_mv(int l) { return l == kLayoutSplitMv || l == kLayoutSplitMvChild; }
-__host__ __device__ constexpr bool layout_child(int l) { return l == kLayoutSplitMvChild; }
-__host__ __device__ constexpr bool layout_arr(int l) { return l == kLayoutSplitArr; }
-
-template <typename Id>
-__host__ __device__ inline size_t lex_split_smem_bytes(int n, int layout) {
-    size_t b = ((size_t)n * sizeof(Id) + 15) & ~size_t(15);
-    b += ((size_t)((n + 31) / 32) * sizeof(uint32_t) + 15) & ~size_t(15);
-    if (layout_mv(layout)) b += ((size_t)((n + 1) / 2) * sizeof(uint32_t) + 15) & ~size_t(15);
-    if (layout_arr(layout)) b += ((size_t)((n + 31) / 32) * sizeof(uint32_t) + 15) & ~size_t(15);
-    if (layout_child(layout)) b += ((size_t)n * sizeof(Id) + 15) & ~size_t(15);
+    if (state != kStateGlobal) b += wn * 32 * 4;       // keys
+    if (state == kStateSmem) b += wn * 32 * 2 * 2;     // perm and its scratch copy
     return b;
 }
+__host__ __device__ inline size_t panel_sort_bytes(int cap) { return (size_t)cap * 12; }
 
-template <typename Id>
-__host__ __device__ inline size_t lex_split_global_bytes(int n, int layout) {
-    using Sz = typename IdTraits<Id>::Sz;
-    const size_t child = layout_child(layout) ? 0 : 1;
-    const size_t b = (size_t)n * sizeof(Sz) + (size_t)n * sizeof(Id) * (1 + child) + (size_t)(n + 1) * sizeof(Id) * 2;
+// Workspace bytes per CTA.
+__host__ __device__ inline size_t panel_global_bytes(int n, int state) {
+    const size_t nv = (size_t)(n + 31) / 32 * 32;
+    const size_t b = state == kStateSmem ? 0 : state == kStatePermGlobal ? nv * 2 * 2 : nv * 4 * 3;
     return (b + 255) & ~size_t(255);
 }
 
-template <typename Id, int LAYOUT>
-__device__ inline LexState<Id> lex_state_carve_split(unsigned char *smem, unsigned char *gmem, int n) {
-    using Sz = typename IdTraits<Id>::Sz;
-    LexState<Id> s;
+template <typename Id>
+struct PanelState {
+    CG_ARR(Id) perm;            // vertices by position
+    CG_ARR(Id) tmp;             // split classes being rewritten
+    CG_ARR(uint32_t) key;       // by key_slot(vertex)
+    CG_ARR(uint32_t) start;     // bit q: a class starts at position q
+    CG_ARR(uint32_t) diff;      // bit q: q's key differs from q - 1's, same class
+    CG_ARR(uint32_t) nz;        // bit q: q's key is not 0 (then: and q's class splits)
+    CG_ARR(uint32_t) flag;      // bit q: q's class splits
+    CG_ARR(uint32_t) numbered;  // bit v: vertex v is numbered
+    CG_ARR(int) dpre;           // differing keys before a word of positions
+    CG_ARR(int) last;           // last class start up to the end of a word of positions
+    CG_ARR(int) next;           // first class start from a word of positions on
+    CG_ARR(int) nzpre;          // moved members of split classes before a word of positions
+    CG_ARR(unsigned long long) comp;   // [cap] moved members: class start, inverted key, list index
+    CG_ARR(uint32_t) lv;        // [cap] their vertices
+    int cap;
+};
+
+// A thread writes the 32 keys of one word of vertices as eight 16-byte pieces;
+// the pieces are rotated by the word's index so that neighbouring threads'
+// pieces fall into different banks.
+__device__ __forceinline__ unsigned key_slot(unsigned v) { return v ^ ((v >> 3) & 0x1Cu); }
+
+template <int STATE>
+__device__ inline PanelState<typename PanelId<STATE>::type> panel_carve(unsigned char *smem, unsigned char *gmem,
+                                                                        int n, int cap) {
+    using Id = typename PanelId<STATE>::type;
+    PanelState<Id> s;
+    const int wn = (n + 31) >> 5;
+    const size_t nv = (size_t)wn * 32;
     unsigned char *q = smem;
-    s.cls = cg_arr(reinterpret_cast<Id *>(q), n, kChkCls);
-    q += ((size_t)n * sizeof(Id) + 15) & ~size_t(15);
-    s.numbered = cg_arr(reinterpret_cast<uint32_t *>(q), (n + 31) / 32, kChkNumbered);
-    q += ((size_t)((n + 31) / 32) * sizeof(uint32_t) + 15) & ~size_t(15);
-    if constexpr (layout_mv(LAYOUT)) {
-        s.mvw = cg_arr(reinterpret_cast<uint32_t *>(q), (n + 1) / 2, kChkMoved);
-        s.mvh = cg_arr(reinterpret_cast<uint16_t *>(q), n, kChkMoved);
-        q += ((size_t)((n + 1) / 2) * sizeof(uint32_t) + 15) & ~size_t(15);
-    }
-    if constexpr (layout_arr(LAYOUT)) {
-        s.arrived = cg_arr(reinterpret_cast<uint32_t *>(q), (n + 31) / 32, kChkMoved);
-        q += ((size_t)((n + 31) / 32) * sizeof(uint32_t) + 15) & ~size_t(15);
-    }
-    s.sz = cg_arr(reinterpret_cast<Sz *>(gmem), n, kChkSize);
-    Id *p = reinterpret_cast<Id *>(gmem + (size_t)n * sizeof(Sz));
-    if constexpr (layout_child(LAYOUT)) {
-        s.child = cg_arr(reinterpret_cast<Id *>(q), n, kChkChild);
+    s.comp = cg_arr(reinterpret_cast<unsigned long long *>(q), cap, kChkSort);
+    q += (size_t)cap * 8;
+    s.lv = cg_arr(reinterpret_cast<uint32_t *>(q), cap, kChkSort);
+    q += (size_t)cap * 4;
+    if constexpr (STATE != kStateGlobal) {
+        s.key = cg_arr(reinterpret_cast<uint32_t *>(q), nv, kChkKey);
+        q += nv * 4;
     } else {
-        s.child = cg_arr(p, n, kChkChild);
-        p += n;
+        s.key = cg_arr(reinterpret_cast<uint32_t *>(gmem), nv, kChkKey);
+        gmem += nv * 4;
     }
-    s.freel = cg_arr(p, n, kChkFree);
-    s.cnext = cg_arr(p + n, n + 1, kChkCnext);
-    s.cprev = cg_arr(p + 2 * (size_t)n + 1, n + 1, kChkCprev);
+    Id *p;
+    if constexpr (STATE == kStateSmem) {
+        p = reinterpret_cast<Id *>(q);
+        q += nv * 2 * 2;
+    } else {
+        p = reinterpret_cast<Id *>(gmem);
+    }
+    s.perm = cg_arr(p, nv, kChkPerm);
+    s.tmp = cg_arr(p + nv, nv, kChkPerm);
+    uint32_t *w = reinterpret_cast<uint32_t *>(q);
+    s.start = cg_arr(w, wn, kChkCls);
+    s.diff = cg_arr(w + wn, wn, kChkSplit);
+    s.nz = cg_arr(w + 2 * (size_t)wn, wn, kChkSplit);
+    s.flag = cg_arr(w + 3 * (size_t)wn, wn, kChkSplit);
+    s.numbered = cg_arr(w + 4 * (size_t)wn, wn, kChkNumbered);
+    int *iw = reinterpret_cast<int *>(w + 5 * (size_t)wn);
+    s.dpre = cg_arr(iw, wn, kChkSplit);
+    s.last = cg_arr(iw + wn, wn, kChkSplit);
+    s.next = cg_arr(iw + 2 * (size_t)wn, wn, kChkSplit);
+    s.nzpre = cg_arr(iw + 3 * (size_t)wn, wn, kChkSplit);
+    s.cap = cap;
     return s;
 }
 
-// Word w of row x as stored, 0 for w >= wn: nothing touches the loaded value
-// here, so the warp does not wait for it until the word is first used
-// (padding bits are cleared there).
-__device__ __forceinline__ uint32_t row_raw(const uint32_t *__restrict__ rows, int stride, int x, int w, int wn) {
-    uint32_t v = 0u;
-#ifdef CG_BOUNDS_CHECK
-    if (w < wn && x < 0) {   // x < n holds when x comes from the state arrays
-        cg_dbg_record(kChkRow, (unsigned long long)(unsigned)x);
-        return 0u;
-    }
-#endif
-    if (w < wn) v = rows[(size_t)x * stride + w];
-    return v;
+// One stage of the 32 x 32 bit transpose: blocks of S bits exchanged between
+// r[k] and r[k + S].
+template <int S, uint32_t M>
+__device__ __forceinline__ void transpose_stage(uint32_t (&r)[32]) {
+#pragma unroll
+    for (int k = 0; k < 32; ++k)
+        if (!(k & S)) {
+            const uint32_t a = r[k], b = r[k + S];
+            if constexpr (S == 16) {
+                r[k] = __byte_perm(a, b, 0x5410);
+                r[k + S] = __byte_perm(a, b, 0x7632);
+            } else if constexpr (S == 8) {
+                r[k] = __byte_perm(a, b, 0x6240);
+                r[k + S] = __byte_perm(a, b, 0x7351);
+            } else {
+                r[k] = (a & M) | ((b << S) & ~M);
+                r[k + S] = ((a >> S) & M) | (b & ~M);
+            }
+        }
+}
+// out[v] bit j = in[j] bit v
+__device__ __forceinline__ void transpose32(uint32_t (&r)[32]) {
+    transpose_stage<16, 0u>(r);
+    transpose_stage<8, 0u>(r);
+    transpose_stage<4, 0x0F0F0F0Fu>(r);
+    transpose_stage<2, 0x33333333u>(r);
+    transpose_stage<1, 0x55555555u>(r);
 }
 
-// One CTA computes the LexBFS order of one graph.  rows/stride address the
-// adjacency (global memory, or a compact shared-memory copy).  parent may be
-// null; otherwise it receives p(v) (-1 when v has no earlier neighbour):
-// under kParentMoves as parent[v], under kParentPivots as parent[i] =
-// p(order[i]) or kParentUnresolved.  lpw >= LPW threads
-// share each row word (thread t takes bit slice t % lpw of word t / lpw +
-// k * T / lpw), which shortens the serial bit loop; lpw grows while T / lpw
-// still covers the row.
-// MV: where the moved counts live: 0 in the packed size words, 1 in the
-// 16-bit counts of st.mvw (split layouts 2, 3), 2 in the packed size words
-// with the allocator elected by st.arrived (split layout 5).
-template <typename Id, int T, int WPT, int LPW, int MV = 0>
-__device__ void lexbfs_cta(const uint32_t *__restrict__ rows, int stride, int n, LexState<Id> st,
-                           LexScalars *sc, int32_t *__restrict__ order, int32_t *__restrict__ pos,
-                           int32_t *__restrict__ parent, int pmode = kParentMoves,
-                           uint32_t *__restrict__ emask = nullptr, int32_t *__restrict__ cpar = nullptr) {
-    using Tr = IdTraits<Id>;
-    using Sz = typename Tr::Sz;
-    const Id kNumbered = (Id)~(Id)0;
-    const Id kNone = (Id)(kNumbered - 1);
-    const int t = threadIdx.x;
-    if (n <= 0) return;
-    const int wn = (n + 31) >> 5;
-    // lanes per word: at least LPW, more while the row still has a word slot
-    // per thread group, so short rows spread their bits over all threads
-    int lpw = LPW;
-    while (lpw < 32 && T / (lpw * 2) >= wn) lpw *= 2;
-    const int kGroups = T / lpw;                // word slots per k
-    const int kSlice = 32 / lpw;                // bits per thread
-    const int wt = t / lpw;
-    const uint32_t part = lpw == 1 ? 0xFFFFFFFFu
-                                   : ((kSlice == 32 ? 0xFFFFFFFFu : ((1u << kSlice) - 1u)) << ((t % lpw) * kSlice));
-    const Id HEAD = (Id)n;
-    const uint32_t lastmask = (n & 31) ? ((1u << (n & 31)) - 1u) : 0xFFFFFFFFu;
-
-    for (int v = t; v < n; v += T) {
-        st.cls[v] = 0;
-        if (parent && pmode == kParentMoves) parent[v] = -1;
-    }
-    for (int k = t; k < n - 1; k += T) st.freel[k] = (Id)(k + 1);
-    for (int w = t; w < wn; w += T) st.numbered[w] = 0u;
-    if constexpr (MV == 1)
-        for (int w = t; w < (n + 1) / 2; w += T) st.mvw[w] = 0u;
-    if constexpr (MV == 2)
-        for (int w = t; w < (n + 31) / 32; w += T) st.arrived[w] = 0u;
-    if (t == 0) {
-        st.sz[0] = (Sz)n;
-        st.cnext[HEAD] = 0;
-        st.cprev[0] = HEAD;
-        st.cnext[0] = kNone;
-        sc->free_top = n - 1;
-        sc->front_min[0] = sc->front_min[1] = kNoVertex;
-        sc->second_min[0] = sc->second_min[1] = kNoVertex;
-        sc->split[0] = sc->split[1] = 0u;
-        if (cpar) cpar[0] = -1;   // class 0 (all vertices) has no numbered neighbour
-    }
-    uint32_t rA[WPT], rB[WPT], rC[WPT], amask[WPT];   // previous / current / next pivot row, as loaded
-    int x = 0;
+// Eight neighbouring 16- or 32-bit entries (16-byte aligned).
+__device__ __forceinline__ void panel_load8(const uint16_t *p, uint16_t (&v)[8]) {
+    const uint4 a = *reinterpret_cast<const uint4 *>(p);
+    const uint32_t x[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
-    for (int k = 0; k < WPT; ++k) {
-        const int w = k * kGroups + wt;
-        rB[k] = row_raw(rows, stride, x, w, wn);
-        rA[k] = 0u;
-        rC[k] = 0u;
-        amask[k] = 0u;
+    for (int e = 0; e < 8; ++e) v[e] = (uint16_t)(x[e >> 1] >> (16 * (e & 1)));
+}
+__device__ __forceinline__ void panel_load8(const uint32_t *p, uint32_t (&v)[8]) {
+    const uint4 a = reinterpret_cast<const uint4 *>(p)[0], b = reinterpret_cast<const uint4 *>(p)[1];
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+}
+
+__device__ __forceinline__ uint32_t lanes_below(int lane) { return (1u << lane) - 1u; }
+__device__ __forceinline__ uint32_t low_bits(int k) { return k >= 32 ? 0xFFFFFFFFu : (1u << k) - 1u; }
+
+// How many window vertices are visited in window order (every warp computes
+// it).  Lane z's turn comes after lanes 0..z-1 if no later vertex of its class
+// has a larger label with respect to them.  A lexicographic >= over lanes 0..z
+// also holds over lanes 0..z-1, so as long as every lane's label is >= the next
+// one's in its class, the later ones need no comparison; a lane with a larger
+// label than the one before it is compared with all before it.  Lanes of a
+// class that goes on beyond the window (straddle) are also compared with ub,
+// the largest label out there.  *order_fails: the first lane that is not
+// visited in order fails inside the window, not against ub.
+__device__ __forceinline__ int panel_in_order(int lane, int w2, uint32_t starts, bool straddle, uint32_t adj,
+                                              uint32_t ub, bool *order_fails) {
+    const uint32_t prefix = lanes_below(lane), above = starts & (0xFFFFFFFEu << lane);
+    auto loses = [&](uint32_t other) {   // label of lane < label of the other, over lanes 0..lane-1
+        const uint32_t d = (adj ^ other) & prefix;
+        return d != 0u && !(adj & d & (0u - d));
+    };
+    const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, adj, 1);
+    const uint32_t f1 = __ballot_sync(0xFFFFFFFFu, straddle && lane < w2 && !above && loses(ub));
+    uint32_t f0 = 0u;
+    for (uint32_t larger = __ballot_sync(0xFFFFFFFFu, lane + 1 < w2 && !((starts >> lane) & 2u) && loses(next)); larger;
+         larger &= larger - 1u) {
+        const int y = __ffs(larger);   // the lane after the one that loses to it
+        const uint32_t other = __shfl_sync(0xFFFFFFFFu, adj, y);
+        f0 |= __ballot_sync(0xFFFFFFFFu, lane < y && !(above & low_bits(y + 1)) && loses(other));
     }
-    Id pending_free = kNone;
-    int par_x = -1;   // p(x) of the current pivot (thread 0, kParentPivots)
+    const uint32_t f = f0 | f1 | ~low_bits(w2);
+    const int r = f ? __ffs(f) - 1 : 32;
+    *order_fails = r < w2 && ((f0 >> r) & 1u);
+    return r;
+}
+
+// LexBFS of the window by one warp.  Lane k holds window vertex k's adjacency
+// mask; starts has the first lane of every class; straddle: the last class
+// continues beyond the window, and outside(j) = bit j of ub says whether
+// pivot j may be adjacent to a member out there.  Returns the number of pivots;
+// mypos = this lane's index among them (-1: not taken), la = the index of its
+// last adjacent pivot before it (-1: none).
+__device__ __forceinline__ int panel_solve(int lane, int w2, uint32_t starts, bool straddle, uint32_t adj, uint32_t ub,
+                                           int *mypos_out, int *la_out) {
+    uint32_t undone = low_bits(w2);
+    starts &= undone;
+    const uint32_t cs = straddle ? undone & (0xFFFFFFFFu << (31 - __clz(starts))) : 0u;
+    uint32_t key = 0u, front = 0u, fkey = 0u, ubkey = 0u, cls = 0u;
+    int r = 0, mypos = -1, la = -1;
+    while (undone) {
+        if (!front) {   // the top class's members with the largest label
+            if (!(cls & undone)) {
+                const int l = __ffs(undone) - 1;
+                const uint32_t above = starts & (0xFFFFFFFEu << l);
+                cls = undone & (above ? (above & (0u - above)) - 1u : 0xFFFFFFFFu) & (0xFFFFFFFFu << l);
+            }
+            const uint32_t cand = cls & undone;
+            const bool in = (cand >> lane) & 1u;
+            fkey = __reduce_max_sync(0xFFFFFFFFu, in ? key : 0u);
+            front = __ballot_sync(0xFFFFFFFFu, in && key == fkey);
+            if ((cls & cs) && fkey < ubkey) break;
+        }
+        const int x = __ffs(front) - 1;
+        const uint32_t bit = (adj >> x) & 1u;
+        const uint32_t a = __ballot_sync(0xFFFFFFFFu, bit);
+        if (lane == x) mypos = r;
+        undone &= ~(1u << x);
+        front &= ~(1u << x);
+        if (bit && ((undone >> lane) & 1u)) la = r;
+        key = 2u * key + bit;
+        ubkey = 2u * ubkey + ((ub >> x) & 1u);
+        ++r;
+        if (front) {
+            const uint32_t f2 = front & a;
+            fkey = 2u * fkey + (f2 ? 1u : 0u);
+            if (f2) front = f2;
+            if ((cls & cs) && fkey < ubkey) break;
+        }
+    }
+    *mypos_out = mypos;
+    *la_out = la;
+    return r;
+}
+
+// Block-wide exclusive scans, one value each per thread: the sum of a, and with
+// MINMAX the maximum of b over the threads before and the minimum of c over the
+// threads after.  Returns the sum of all a.  Two barriers.
+template <int T, bool MINMAX>
+__device__ __forceinline__ int panel_scan(PanelScalars *sc, int &a, int &b, int &c) {
+    constexpr int NW = T / 32;
+    constexpr int kBig = 0x7FFFFFFF;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int ia = a, ib = b, ic = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int ua = __shfl_up_sync(0xFFFFFFFFu, ia, o);
+        if (lane >= o) ia += ua;
+        if constexpr (MINMAX) {
+            const int ub = __shfl_up_sync(0xFFFFFFFFu, ib, o);
+            const int dc = __shfl_down_sync(0xFFFFFFFFu, ic, o);
+            if (lane >= o) ib = max(ib, ub);
+            if (lane + o < 32) ic = min(ic, dc);
+        }
+    }
+    if (lane == 31) {
+        sc->scan[0][warp] = ia;
+        if constexpr (MINMAX) sc->scan[1][warp] = ib;
+    }
+    if constexpr (MINMAX) {
+        if (lane == 0) sc->scan[2][warp] = ic;
+        ib = __shfl_up_sync(0xFFFFFFFFu, ib, 1);
+        ic = __shfl_down_sync(0xFFFFFFFFu, ic, 1);
+        if (lane == 0) ib = -1;
+        if (lane == 31) ic = kBig;
+    }
+    __syncthreads();
+    const int wa = lane < NW ? sc->scan[0][lane] : 0;
+    const int total = __reduce_add_sync(0xFFFFFFFFu, wa);
+    a = ia - a + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? wa : 0);
+    if constexpr (MINMAX) {
+        b = max(ib, __reduce_max_sync(0xFFFFFFFFu, lane < warp ? sc->scan[1][lane] : -1));
+        c = min(ic, __reduce_min_sync(0xFFFFFFFFu, lane > warp && lane < NW ? sc->scan[2][lane] : kBig));
+    }
+    __syncthreads();
+    return total;
+}
+
+// Sorts a[0..p), p a power of two, ascending.  Pair exchanges at distances up
+// to 32 stay inside a warp's 64 elements and need no CTA barrier.
+template <int T>
+__device__ __forceinline__ void panel_sort(unsigned long long *a, int p) {
+    for (int k = 2; k <= p; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int e = threadIdx.x; e < p / 2; e += T) {
+                const int lo = ((e & ~(j - 1)) << 1) | (e & (j - 1)), hi = lo | j;
+                const unsigned long long x = a[lo], y = a[hi];
+                if ((x > y) == ((lo & k) == 0)) {
+                    a[lo] = y;
+                    a[hi] = x;
+                }
+            }
+            const int nj = j > 1 ? j >> 1 : k;
+            if (j > 32 || nj > 32) __syncthreads();
+            else __syncwarp();
+        }
+    __syncthreads();
+}
+
+// E_b from the numbered mask (padding words are zero).
+template <int T, typename Arr>
+__device__ __forceinline__ void panel_write_mask(uint32_t *emask, int b, int n, const Arr &numbered) {
+    const int wn = (n + 31) >> 5, es = mask_stride(n);
+    uint32_t *e = emask + (size_t)b * es;
+    for (int w = threadIdx.x; w < es; w += T) e[w] = w < wn ? numbered[w] : 0u;
+}
+
+// One CTA computes the LexBFS order of one graph (rows: n rows of `stride`
+// words in global memory).  order gets the vertices by position; pos (nullable)
+// its inverse; ppos (nullable) p(order[i]) by position (-1: none), exact; emask
+// (nullable) the masks E_b, b >= 1, rows of mask_stride(n) words.
+template <int STATE, int T>
+__device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int n,
+                              const PanelState<typename PanelId<STATE>::type> &st, PanelScalars *sc,
+                              int32_t *__restrict__ order, int32_t *__restrict__ pos, int32_t *ppos, uint32_t *emask) {
+    using Id = typename PanelId<STATE>::type;
+    constexpr int NW = T / 32;
+    constexpr unsigned kAll = 0xFFFFFFFFu;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int wn = (n + 31) >> 5;
+
+    for (int q = t; q < 32 * wn; q += T) st.perm[q] = (Id)q;   // positions past n too: they are read in eights
+    for (int w = t; w < wn; w += T) {
+        st.start[w] = w == 0 ? 1u : 0u;
+        st.diff[w] = 0u;
+        st.nz[w] = 0u;
+        st.numbered[w] = 0u;
+    }
+    if (t == 0 && ppos) ppos[0] = -1;
     __syncthreads();
 
-    // adds k to class c's moved count; true for the first arrival of the step
-    // (that thread allocates for the class)
-    auto moved_add = [&](Id c, unsigned k) -> bool {
-        if constexpr (MV == 1) {
-            const unsigned sh = (unsigned)(c & 1) << 4;
-            return ((atomicAdd(&st.mvw[c >> 1], k << sh) >> sh) & 0xFFFFu) == 0u;
-        } else if constexpr (MV == 2) {
-            atomicAdd(&st.sz[c], (Sz)k << Tr::kShift);   // no return value: the chain does not wait for it
-            const uint32_t bit = 1u << (c & 31);
-            return (atomicOr(&st.arrived[c >> 5], bit) & bit) == 0u;
-        } else {
-            return (atomicAdd(&st.sz[c], (Sz)k << Tr::kShift) >> Tr::kShift) == 0;
-        }
-    };
-    auto step = [&](const int i, uint32_t (&row_prev)[WPT], uint32_t (&row_cur)[WPT],
-                    uint32_t (&row_nxt)[WPT]) -> bool {
-        const int slot = i & 1;
-        const Id f = st.cnext[HEAD];
-        const Id g = st.cnext[f];
-        const Sz fsz = MV == 1 ? st.sz[f] : st.sz[f] & Tr::kMask;  // still counts x
-        // uniform shortcuts: when the previous step split no class, every class
-        // that moved kept its id and the relabel is a no-op; when f is the only
-        // class, every unnumbered neighbour of x is in f and a warp adds its
-        // count to f with one atomic (cliques take this path at every step)
-        const bool relabel = sc->split[slot ^ 1] != 0u;
-        const bool single = g == kNone;
-        // parent of a pivot scanned from g (thread 0; used after barrier A, so the load overlaps phase S)
-        const int cpar_g = t == 0 && cpar && g != kNone ? cpar[g] : kParentUnresolved;
-
-        // E_b = the vertices numbered before x, written at every step 32 b
-        // (x's own bit may already be set by a thread of phase S, so it is cleared)
-        if (emask && (i & 31) == 0 && i > 0) {
-            const int xw = x >> 5;
-            uint32_t *eb = emask + (size_t)(i >> 5) * mask_stride(n);
-            for (int w = t; w < mask_stride(n); w += T) {   // padding words past ceil(n/32) are zero
-                const uint32_t nb = w < wn ? st.numbered[w] : 0u;
-                eb[w] = w == xw ? nb & ~(1u << (x & 31)) : nb;
-            }
-        }
-        // ---- phase S: deferred relabel, number x, split by N(x)
-        if (t == 0) {
-            if (pending_free != kNone) {
-                st.freel[sc->free_top] = pending_free;
-                sc->free_top += 1;
-                pending_free = kNone;
-            }
-            order[i] = x;
-            if (pos) pos[x] = i;
-            if (parent && pmode == kParentPivots) parent[i] = par_x;
-        }
+    int eb = 0;   // E_eb is to be written at the start of the next panel (0: none)
+    int i = 0;    // numbered vertices
+    while (i < n) {
+        const int w2 = min(32, n - i);
+        const int vk = lane < w2 ? (int)st.perm[i + lane] : 0;
+        // the window's classes (read before warp 0 may set a start for the next panel)
+        const uint32_t starts =
+            __funnelshift_r(st.start[i >> 5], (i >> 5) + 1 < wn ? st.start[(i >> 5) + 1] : 0u, i & 31) & low_bits(w2);
+        const bool straddle = i + w2 < n && !((st.start[(i + w2) >> 5] >> ((i + w2) & 31)) & 1u);
+        int cp = -1;   // warp 0: the classes' last adjacent pivots, requested early
+        if (warp == 0 && ppos && lane < w2) cp = __ldcg(ppos + i + lane);
+        if (eb > 0) panel_write_mask<T>(emask, eb, n, st.numbered);
+        // ---- keys: a word of vertices per thread and pass
+        for (int wb = warp * 32; wb < wn; wb += T) {
+            const int w = wb + lane;
+            const bool on = w < wn && st.numbered[w] != kAll;   // some vertex still to come
+            if (!__any_sync(kAll, on)) continue;
+            uint32_t r[32];
 #pragma unroll
-        for (int k = 0; k < WPT; ++k) {
-            const int w = k * kGroups + wt;
-            uint32_t am = 0u;
-            if (w < wn) {
-                const uint32_t prev = row_prev[k];
-                uint32_t nb = st.numbered[w];
-                // relabel pass: vertices moved by the previous pivot take their new class
-                uint32_t bits = relabel ? prev : 0u;
-                while (bits) {
-                    const int y = (w << 5) + (__ffs(bits) - 1);
-                    bits &= bits - 1;
-                    st.cls[y] = st.child[st.cls[y]];
+            for (int j = 0; j < 32; ++j) {
+                const int vj = __shfl_sync(kAll, vk, j);
+                r[j] = on && j < w2 ? rows[(size_t)vj * stride + w] : 0u;
+            }
+            transpose32(r);
+            if (on) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    *reinterpret_cast<uint4 *>(&st.key[32 * w + ((c ^ (w & 7)) << 2)]) =
+                        make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+            }
+        }
+        if (t == 0) sc->any = 0;
+        __syncthreads();
+        if (warp == 0 && eb > 0 && lane < sc->r && i - sc->r + lane >= 32 * eb)   // the last panel's pivots after E_eb
+            atomicOr(&st.numbered[sc->piv[lane] >> 5], 1u << (sc->piv[lane] & 31));
+
+        // ---- the pivots: window vertices 0..r-1 in order, or what warp 0 finds
+        const uint32_t adj = lane < w2 ? st.key[key_slot(vk)] : 0u;   // window vertex `lane` in the window
+        int mypos = -1, la = -1;   // warp 0
+        auto commit = [&](int r) {
+            const bool ident = __ballot_sync(kAll, mypos >= 0 && mypos != lane) == 0u;
+            const uint32_t taken = __ballot_sync(kAll, mypos >= 0), left = low_bits(w2) & ~taken;
+            const int own = __shfl_sync(kAll, cp, 31 - __clz((starts | 1u) & low_bits(lane + 1)));   // its class's value
+            const int cl = left ? __ffs(left) - 1 : w2 - 1;   // a member of the class that goes on at position i + r
+            const int cpl = __shfl_sync(kAll, own, cl);
+            if (mypos >= 0) sc->piv[mypos] = vk;
+            if (!ident) {
+                const int dest = mypos >= 0 ? mypos : r + __popc(left & lanes_below(lane));
+                if (lane < w2) st.perm[i + dest] = (Id)vk;
+                sc->bit[lane] = mypos >= 0 ? 0x80000000u >> mypos : 0u;
+            }
+            __syncwarp();
+            if (mypos >= 0) sc->par[mypos] = la >= 0 ? sc->piv[la] : own;
+            if (lane == 0) {
+                const int i2 = i + r;
+                int set = -1;
+                if (i2 < n && !((st.start[i2 >> 5] >> (i2 & 31)) & 1u)) {
+                    st.start[i2 >> 5] |= 1u << (i2 & 31);
+                    set = i2;
+                    if (ppos) ppos[i2] = cpl;
                 }
-                uint32_t rw = row_cur[k];   // first use of the pivot row's word
-                if (w == wn - 1) rw &= lastmask;
-                const uint32_t cur = rw & part & ~nb;  // unnumbered neighbours of x
-                // split pass: count moved members per class; a lane's first moved
-                // member of the top class (or of the next one) is its pivot candidate
-                bits = single ? 0u : cur;
-                if (single && parent && pmode == kParentMoves)
-                    for (uint32_t pb = cur; pb; pb &= pb - 1) parent[(w << 5) + (__ffs(pb) - 1)] = x;
-                bool f_done = false, g_done = false;
-                while (bits) {
-                    const int b = __ffs(bits) - 1;
-                    const uint32_t bit = 1u << b;
-                    bits &= bits - 1;
-                    const int y = (w << 5) + b;
-                    const Id c = st.cls[y];
-                    if (moved_add(c, 1u)) am |= bit;
-                    if (!f_done && c == f) {
-                        atomicMin(&sc->front_min[slot], (unsigned)y);
-                        f_done = true;
-                    } else if (!g_done && c == g) {
-                        atomicMin(&sc->second_min[slot], (unsigned)y);
-                        g_done = true;
+                sc->set_start = set;
+                sc->r = r;
+                sc->pivmask = taken;
+                sc->ident = ident ? 1 : 0;
+            }
+        };
+        auto commit_in_order = [&](int r) {
+            mypos = lane < r ? lane : -1;
+            const uint32_t before = adj & lanes_below(lane);
+            la = before ? 31 - __clz(before) : -1;
+            commit(r);
+        };
+        uint32_t ub = kAll;
+        bool order_fails;
+        int r = panel_in_order(lane, w2, starts, straddle, adj, ub, &order_fails);
+        bool ident = true;
+        if (r < w2 && r < kPanelFew) {   // too few (the same in every warp)
+            if (!order_fails) {          // stopped by the class that goes on beyond the window: look at it
+                if (t == 0) {
+                    sc->cend = n;
+                    sc->ub = 0u;
+                }
+                __syncthreads();
+                const int q0 = i + w2;
+                for (int w = (q0 >> 5) + t; w < wn; w += T) {
+                    const uint32_t b = st.start[w] & (w == (q0 >> 5) ? kAll << (q0 & 31) : kAll);
+                    if (b) {
+                        atomicMin(&sc->cend, 32 * w + __ffs(b) - 1);
+                        break;
                     }
-                    if (parent && pmode == kParentMoves) parent[y] = x;
                 }
-                if (w == (x >> 5) && ((part >> (x & 31)) & 1u)) {
-                    st.cls[x] = kNumbered;
-                    st.numbered[w] = nb | (1u << (x & 31));
-                }
-                row_cur[k] = cur;
+                __syncthreads();
+                const int ce = sc->cend;
+                uint32_t any = 0u;
+                for (int q = q0 + t; q < ce; q += T) any |= st.key[key_slot(st.perm[q])];
+                any = __reduce_or_sync(kAll, any);
+                if (lane == 0 && any) atomicOr(&sc->ub, any);
+                __syncthreads();
+                ub = sc->ub;
+                r = panel_in_order(lane, w2, starts, straddle, adj, ub, &order_fails);
             }
-            if (single) {   // warp-uniform: the warp's count of f's moved members in one atomic
-                const uint32_t cur = w < wn ? row_cur[k] : 0u;
-                const unsigned total = __reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(cur));
-                const unsigned lanes = __ballot_sync(0xFFFFFFFFu, cur != 0u);
-                if (lanes && (t & 31) == __ffs(lanes) - 1) {   // the warp's lowest moved vertex
-                    if (moved_add(f, total)) am = cur & (0u - cur);   // first arrival allocates
-                    atomicMin(&sc->front_min[slot], (unsigned)((w << 5) + __ffs(cur) - 1));
-                }
-            }
-            amask[k] = am;
+            ident = !(order_fails && r < kPanelFew);
         }
-        __syncthreads();  // A
-
-        // ---- phase D: next pivot (uniform decision)
-        const unsigned fmin = sc->front_min[slot];
-        const unsigned gmin = sc->second_min[slot];
-        const bool fempty = (fsz == 1);
-        int mode;  // 0 pivot known, 1 scan class f, 2 scan class g, 3 finished
-        unsigned xn = 0;
-        Id target = 0;
-        if (fmin != kNoVertex) {
-            mode = 0;
-            xn = fmin;
-        } else if (!fempty) {
-            mode = 1;
-            target = f;
-        } else if (g == kNone) {
-            mode = 3;
-        } else if (gmin != kNoVertex) {
-            mode = 0;
-            xn = gmin;
+        uint32_t pm = low_bits(r);
+        if (ident) {
+            if (warp == 0) commit_in_order(r);
         } else {
-            mode = 2;
-            target = g;
-        }
-        // a moved pivot's parent is x; one scanned from f shares x's; one from g has g's
-        if (t == 0) par_x = mode == 0 ? x : mode == 1 && cpar ? par_x : cpar_g;
-        if (mode == 0) {
-#pragma unroll
-            for (int k = 0; k < WPT; ++k) row_nxt[k] = row_raw(rows, stride, (int)xn, k * kGroups + wt, wn);
+            __syncthreads();   // every warp has read ub
+            if (warp == 0) commit(panel_solve(lane, w2, starts, straddle, adj, ub, &mypos, &la));
+            __syncthreads();
+            r = sc->r;
+            pm = sc->pivmask;
+            ident = sc->ident != 0;
         }
 
-        // ---- phase A: allocate / link split classes
+        // ---- classes whose members' keys differ: a lane compares eight neighbouring positions
+        int i2;
+        // a key's bits in pivot order, the first pivot's highest
+        auto pivot_key = [&](uint32_t k) -> uint32_t {
+            if (ident) return __brev(k);
+            uint32_t v = 0u;
 #pragma unroll
-        for (int k = 0; k < WPT; ++k) {
-            const int w = k * kGroups + wt;
-            uint32_t am = amask[k];
-            while (am) {
-                const int y = (w << 5) + (__ffs(am) - 1);
-                am &= am - 1;
-                const Id c = st.cls[y];  // class before this step's move (relabel is deferred)
-                Sz mv, size;
-                if constexpr (MV == 1) {
-                    mv = (st.mvw[c >> 1] >> ((c & 1) << 4)) & 0xFFFFu;
-                    size = st.sz[c] - (c == f ? 1 : 0);
-                    st.mvh[c] = 0;   // the moved count restarts (the other half of the word is another class's)
-                } else {
-                    if constexpr (MV == 2) atomicAnd(&st.arrived[c >> 5], ~(1u << (c & 31)));
-                    const Sz s = st.sz[c];
-                    mv = s >> Tr::kShift;
-                    size = (s & Tr::kMask) - (c == f ? 1 : 0);
+            for (int b = 0; b < 8; ++b) v |= sc->tab[b][(k >> (4 * b)) & 15u];
+            return v;
+        };
+        for (;;) {
+            i2 = i + r;
+            if (!ident)
+                for (int e = t; e < 128; e += T) {
+                    uint32_t v = 0u;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+                        if ((e >> b) & 1) v |= sc->bit[((e >> 4) << 2) + b];
+                    sc->tab[e >> 4][e & 15] = v;
                 }
-                if (mv == size) {
-                    st.child[c] = c;
-                    st.sz[c] = size;
-                    if (cpar) cpar[c] = x;
-                    if (fempty && c == g) {
-                        st.cnext[HEAD] = g;
-                        st.cprev[g] = HEAD;
+            bool differ = false;
+            for (int c = (i2 & ~255) + warp * 256; c < n; c += T * 8) {
+                const int q0 = c + 8 * lane;
+                uint32_t k[8], kp = 0u;
+                if (q0 < n) {
+                    Id v[8];
+                    panel_load8(&st.perm[q0], v);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) k[e] = st.key[key_slot(v[e])] & pm;
+                    if (lane == 0 && q0 > i2) kp = st.key[key_slot(st.perm[q0 - 1])] & pm;
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) k[e] = 0u;
+                }
+                const uint32_t up = __shfl_up_sync(kAll, k[7], 1);
+                if (lane > 0) kp = up;
+                if (q0 < n) {
+                    uint32_t dm = 0u, nm = 0u;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        dm |= (k[e] != (e ? k[e - 1] : kp) ? 1u : 0u) << e;
+                        nm |= (k[e] ? 1u : 0u) << e;
+                    }
+                    uint32_t live = q0 >= i2 ? 0xFFu : q0 + 8 > i2 ? 0xFFu << (i2 - q0) : 0u;   // positions i2..n-1
+                    if (q0 + 8 > n) live &= low_bits(n - q0);
+                    nm &= live;
+                    if (q0 <= i2) live &= live - 1u;   // i2 itself starts a class
+                    dm &= live & ~(uint32_t)reinterpret_cast<const uint8_t *>(&st.start[q0 >> 5])[(q0 >> 3) & 3];
+                    reinterpret_cast<uint8_t *>(&st.diff[q0 >> 5])[(q0 >> 3) & 3] = (uint8_t)dm;
+                    reinterpret_cast<uint8_t *>(&st.nz[q0 >> 5])[(q0 >> 3) & 3] = (uint8_t)nm;
+                    differ |= dm != 0u;
+                }
+            }
+            if (__any_sync(kAll, differ) && lane == 0) sc->any = 1;
+            __syncthreads();
+            if (!sc->any) break;
+            const int pw = i2 >> 5;
+
+            // ---- positions of the classes that split (thread t: words [wa, wb) of positions)
+            const int kw = (wn + T - 1) / T, wa = min(t * kw, wn), wb = min(wa + kw, wn);
+            int ds = 0, lm = -1, nm = 0x7FFFFFFF;
+            for (int w = wa; w < wb; ++w) {
+                const uint32_t b = st.start[w];
+                if (w >= pw) ds += __popc(st.diff[w]);
+                if (b) {
+                    lm = 32 * w + 31 - __clz(b);
+                    if (nm == 0x7FFFFFFF) nm = 32 * w + __ffs(b) - 1;
+                }
+            }
+            const int dtotal = panel_scan<T, true>(sc, ds, lm, nm);
+            for (int w = wa; w < wb; ++w) {
+                const uint32_t b = st.start[w];
+                st.dpre[w] = ds;
+                if (w >= pw) ds += __popc(st.diff[w]);
+                if (b) lm = 32 * w + 31 - __clz(b);
+                st.last[w] = lm;
+            }
+            nm = min(nm, n);
+            for (int w = wb - 1; w >= wa; --w) {
+                const uint32_t b = st.start[w];
+                if (b) nm = 32 * w + __ffs(b) - 1;
+                st.next[w] = nm;
+            }
+            if (t == 0) sc->nz_max = 0;
+            __syncthreads();
+            auto diffs_before = [&](int q) -> int {
+                if (q >= n) return dtotal;
+                const int w = q >> 5;
+                return w < pw ? 0 : st.dpre[w] + __popc(st.diff[w] & lanes_below(q & 31));
+            };
+            int nzs = 0;
+            for (int w = wa; w < wb; ++w) {
+                uint32_t f = 0u;
+                if (w >= pw) {
+                    const uint32_t b = st.start[w], d = st.diff[w];
+                    const int nx = w + 1 < wn ? st.next[w + 1] : n;
+                    const uint32_t lead = b ? (b & (0u - b)) - 1u : kAll;   // before the word's first start
+                    uint32_t tail = 0u;
+                    if (lead && w > 0 &&
+                        diffs_before(b ? 32 * w + __ffs(b) - 1 : nx) > diffs_before(st.last[w - 1]))
+                        f |= lead;
+                    if (b) {
+                        tail = kAll << (31 - __clz(b));
+                        if (diffs_before(nx) > diffs_before(32 * w + 31 - __clz(b))) f |= tail;
+                    }
+                    uint32_t inner = d & ~lead & ~tail;   // classes inside the word
+                    while (inner) {
+                        const int q = __ffs(inner) - 1;
+                        const uint32_t lo = 31 - __clz(b & lanes_below(q + 1)), up = b & (0xFFFFFFFEu << q);
+                        const uint32_t m = ((up & (0u - up)) - 1u) & (kAll << lo);
+                        f |= m;
+                        inner &= ~m;
+                    }
+                    st.nz[w] &= f;
+                    nzs += __popc(st.nz[w]);
+                }
+                st.flag[w] = f;
+            }
+            int unused0 = 0, unused1 = 0;
+            const int m = panel_scan<T, false>(sc, nzs, unused0, unused1);
+            if (m > st.cap && r > 1) {   // more to sort than fits: the panel ends after its first pivot
+                r = 1;
+                pm = 1u;
+                if (warp == 0) {
+                    if (!ident && lane < w2) st.perm[i + lane] = (Id)vk;
+                    if (lane == 0) {
+                        if (sc->set_start >= 0) st.start[sc->set_start >> 5] &= ~(1u << (sc->set_start & 31));
+                        sc->any = 0;
+                    }
+                    __syncwarp();
+                    commit_in_order(1);
+                }
+                ident = true;
+                __syncthreads();
+                continue;
+            }
+            for (int w = wa; w < wb; ++w) {
+                st.nzpre[w] = nzs;
+                if (w >= pw) nzs += __popc(st.nz[w]);
+            }
+            __syncthreads();
+            // moved members of split classes before position q (w >= pw); a class's start and end
+            auto moved_before = [&](int q) -> int {
+                return q >= n ? m : st.nzpre[q >> 5] + __popc(st.nz[q >> 5] & lanes_below(q & 31));
+            };
+            auto class_start = [&](int q) -> int {
+                const uint32_t b = st.start[q >> 5] & low_bits((q & 31) + 1);
+                return b ? (q & ~31) + 31 - __clz(b) : st.last[(q >> 5) - 1];
+            };
+            auto class_end = [&](int q) -> int {
+                const uint32_t b = st.start[q >> 5] & (0xFFFFFFFEu << (q & 31));
+                return b ? (q & ~31) + __ffs(b) - 1 : (q >> 5) + 1 < wn ? st.next[(q >> 5) + 1] : n;
+            };
+            // ---- moved members listed, the others shifted to the end of their class
+            for (int w = pw + warp; w < wn; w += NW) {
+                const uint32_t f = st.flag[w];
+                if (!f) continue;
+                const int q = (w << 5) + lane;
+                if (!((f >> lane) & 1u) || q >= n) continue;
+                const Id v = st.perm[q];
+                const int s = class_start(q), e = class_end(q);
+                const int before = moved_before(q), ms = moved_before(s), me = moved_before(e);
+                if ((st.nz[w] >> lane) & 1u) {
+                    if (r == 1) {
+                        st.tmp[s + before - ms] = v;
+                    } else {
+                        const uint32_t pk = pivot_key(st.key[key_slot(v)] & pm);
+                        st.comp[before] = (unsigned long long)s << 44 | (unsigned long long)~pk << 12 | (unsigned)before;
+                        st.lv[before] = v;
+                        if (before == ms) atomicMax(&sc->nz_max, me - ms);
                     }
                 } else {
-                    const int idx = atomicSub(&sc->free_top, 1) - 1;
-                    sc->split[slot] = 1u;
-                    const Id cn = st.freel[idx];
-                    if (cpar) cpar[cn] = x;
-                    st.child[c] = cn;
-                    st.sz[cn] = mv;
-                    st.sz[c] = size - mv;
-                    Id p = st.cprev[c];
-                    if (fempty && p == f) p = HEAD;
-                    st.cnext[p] = cn;
-                    st.cprev[cn] = p;
-                    st.cnext[cn] = c;
-                    st.cprev[c] = cn;
+                    st.tmp[q + me - before] = v;
+                }
+            }
+            __syncthreads();
+            // ---- the moved members in their new order
+            if (r > 1) {
+                if (sc->nz_max <= 64) {   // few per class: every member counts those before it
+                    for (int e = t; e < m; e += T) {
+                        const unsigned long long c = st.comp[e];
+                        const int s = (int)(c >> 44), lo = moved_before(s), hi = moved_before(class_end(s));
+                        int rank = 0;
+                        for (int k = lo; k < hi; ++k) rank += st.comp[k] < c ? 1 : 0;
+                        st.tmp[s + rank] = (Id)st.lv[e];
+                    }
+                } else {
+                    int p = 64;
+                    while (p < m) p <<= 1;
+                    for (int e = m + t; e < p; e += T) st.comp[e] = ~0ull;
+                    __syncthreads();
+                    panel_sort<T>(st.comp, p);
+                    for (int e = t; e < m; e += T) {
+                        const unsigned long long c = st.comp[e];
+                        const int s = (int)(c >> 44);
+                        st.tmp[s + e - moved_before(s)] = (Id)st.lv[c & 0xFFFu];
+                    }
+                }
+                __syncthreads();
+            }
+            // ---- back into perm, with the new boundaries
+            for (int w = pw + warp; w < wn; w += NW) {
+                const uint32_t f = st.flag[w];
+                if (!f) continue;
+                const int q = (w << 5) + lane;
+                const bool on = ((f >> lane) & 1u) && q < n;
+                const uint32_t b = st.start[w];
+                uint32_t k = 0u;
+                if (on) {
+                    const Id v = st.tmp[q];
+                    st.perm[q] = v;
+                    k = st.key[key_slot(v)] & pm;
+                }
+                uint32_t kp = __shfl_up_sync(kAll, k, 1);
+                const bool inside = on && !((b >> lane) & 1u);
+                if (lane == 0 && inside) kp = st.key[key_slot(st.tmp[q - 1])] & pm;
+                const bool fresh = inside && k != kp;
+                const uint32_t nb = __ballot_sync(kAll, fresh);
+                // the members that did not move keep the class's last adjacent pivot
+                if (ppos && fresh && k == 0u) {
+                    const uint32_t le = b & low_bits(lane + 1);
+                    ppos[q] = __ldcg(ppos + (le ? (w << 5) + 31 - __clz(le) : st.last[w - 1]));
+                }
+                __syncwarp();
+                if (lane == 0 && nb) st.start[w] = b | nb;
+            }
+            __syncthreads();
+            break;
+        }
+
+        // ---- the panel's results; every class's last adjacent pivot
+        const int b2 = i2 >> 5;
+        eb = emask && 32 * b2 > i && 32 * b2 < n ? b2 : 0;
+        if (warp == 0 && lane < r) {
+            const int v = sc->piv[lane];
+            order[i + lane] = v;
+            if (pos) pos[v] = i + lane;
+            if (ppos) ppos[i + lane] = sc->par[lane];
+            if (eb == 0 || i + lane < 32 * eb) atomicOr(&st.numbered[v >> 5], 1u << (v & 31));
+        }
+        if (ppos) {
+            for (int q0 = (i2 & ~7) + 8 * t; q0 < n; q0 += 8 * T) {
+                uint32_t b = reinterpret_cast<const uint8_t *>(&st.start[q0 >> 5])[(q0 >> 3) & 3];
+                if (q0 < i2) b &= 0xFFu << (i2 - q0);
+                for (; b; b &= b - 1u) {
+                    const int q = q0 + __ffs(b) - 1;
+                    const uint32_t k = st.key[key_slot(st.perm[q])] & pm;
+                    if (k) ppos[q] = sc->piv[32 - __ffs(pivot_key(k))];
                 }
             }
         }
-        if (t == 0) {
-            if (fmin == kNoVertex) st.sz[f] = fsz - 1;
-            if (fempty) {
-                pending_free = f;
-                if (g == kNone || gmin == kNoVertex) {
-                    st.cnext[HEAD] = g;
-                    if (g != kNone) st.cprev[g] = HEAD;
-                }
-            }
-            sc->front_min[slot ^ 1] = kNoVertex;
-            sc->split[slot ^ 1] = 0u;   // read at the start of this step by every thread (before barrier A)
-            sc->second_min[slot ^ 1] = kNoVertex;
-        }
-        // class scan for the next pivot, overlapping phase A (cls is not written there)
-        if (mode == 1 || mode == 2) {
-            unsigned best = kNoVertex;
-            for (int v = t; v < n; v += T)
-                if (st.cls[v] == target) {
-                    best = (unsigned)v;
-                    break;
-                }
-            best = __reduce_min_sync(0xFFFFFFFFu, best);
-            if ((t & 31) == 0) sc->red[t >> 5] = best;
-        }
-        __syncthreads();  // B
-        if (mode == 3) return false;
-        if (mode != 0) {
-            const unsigned r = (t & 31) < (T / 32) ? sc->red[t & 31] : kNoVertex;
-            xn = __reduce_min_sync(0xFFFFFFFFu, r);
-#pragma unroll
-            for (int k = 0; k < WPT; ++k) row_nxt[k] = row_raw(rows, stride, (int)xn, k * kGroups + wt, wn);
-        }
-        x = (int)xn;
-        return true;
-    };
-    if constexpr (WPT == 1) {
-        // one row word per thread: three registers rotate through the roles
-        // previous / current / next pivot row (the loop is unrolled three
-        // times), so no register copy at the end of a step waits for the next
-        // row's load; the load is first consumed in the next step's split pass,
-        // after its relabel pass (9% faster per step on GB300 at N = 16,384)
-        for (int i = 0; i < n; i += 3) {
-            if (!step(i, rA, rB, rC) || i + 1 >= n) break;
-            if (!step(i + 1, rB, rC, rA) || i + 2 >= n) break;
-            if (!step(i + 2, rC, rA, rB)) break;
-        }
-    } else {   // several words per thread: the rotation would spill, so the rows are copied
-        for (int i = 0; i < n; ++i) {
-            if (!step(i, rA, rB, rC)) break;
-#pragma unroll
-            for (int k = 0; k < WPT; ++k) {
-                rA[k] = rB[k];
-                rB[k] = rC[k];
-            }
-        }
+        i = i2;
+        __syncthreads();
     }
+    if (eb > 0) panel_write_mask<T>(emask, eb, n, st.numbered);
 }
 
 }  // namespace cg

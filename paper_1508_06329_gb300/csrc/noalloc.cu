@@ -104,7 +104,7 @@ extern "C" int cg_chordal_test_dense_noalloc(const cg_dense *g, cg_result *res, 
     if ((rc = lexbfs_dense_plan(n, 0, &plan))) return rc;
     if (plan.gstate_bytes) return set_error(CG_EINVAL, "no-allocation path needs the shared-memory variant");
     int32_t *pos = reinterpret_cast<int32_t *>(scratch + kOffPos);
-    int32_t *parent = reinterpret_cast<int32_t *>(scratch + kOffParent);
+    int32_t *ppos = reinterpret_cast<int32_t *>(scratch + kOffParent);
     int32_t *ord = order ? order : reinterpret_cast<int32_t *>(scratch + kOffOrder);
     unsigned long long *key = reinterpret_cast<unsigned long long *>(scratch + kOffKey);
     int *counter = reinterpret_cast<int *>(scratch + kOffCounter);
@@ -114,9 +114,10 @@ extern "C" int cg_chordal_test_dense_noalloc(const cg_dense *g, cg_result *res, 
     d.words = g->words_per_row;
     d.vbase = 0;
     d.obase = 0;
-    if (n > 0 && (rc = lexbfs_dense_launch(plan, nullptr, d, 1, 1, ord, pos, parent, nullptr, counter, stream)))
-        return rc;
-    // peo_dense_launch resets the key to its "no violation" value before the check
-    if ((rc = peo_dense_launch(nullptr, d, 1, nullptr, n, ord, pos, parent, true, key, num_sms, stream))) return rc;
-    return finalize_launch(nullptr, d, 1, key, ord, parent, res, stream);
+    if (n == 0)
+        return peo_dense_launch(nullptr, d, 1, nullptr, 0, ord, pos, ppos, true, key, num_sms, stream, nullptr, 0,
+                                false, res);
+    // the search sets the witness key to its "no violation" value
+    if ((rc = lexbfs_dense_launch(plan, nullptr, d, 1, 1, ord, pos, ppos, nullptr, counter, stream, key))) return rc;
+    return peo_unit_launch(nullptr, d, 1, n, peo_rows_vec_ok(d), ord, pos, ppos, key, res, stream);
 }

@@ -31,7 +31,6 @@
 #include <vector>
 
 #include "host.h"
-#include "lexbfs_dense.cuh"
 
 namespace cg {
 
@@ -107,12 +106,14 @@ struct Slot {
     bool busy = false;
 };
 
-// Admission estimate for one dense test (order, pos, parent, key, descriptor,
-// result, and the 32-bit search state above 16,384 vertices).  The exact
-// batch size is computed before a batch is admitted.
+// Admission estimate for one dense test (order, pos, parents, key, descriptor,
+// result, and 28 bytes per vertex of search state above 16,384 vertices, more
+// than any state layout takes).  The exact batch size is computed before a
+// batch is admitted.
 size_t dense_need(int n) {
+    const size_t state = ((28 * (size_t)n + 8 + 15) & ~size_t(15)) + (size_t)((n + 31) / 32) * 4;
     return align_up(3 * (size_t)n * 4 + 64 + 16, kAlign) * 2 +
-           (n > 16384 ? align_up(lex_state_bytes<uint32_t>(n), kAlign) : 0);   // covers the split layout too
+           (n > 16384 ? align_up((state + 15) & ~size_t(15), kAlign) : 0);
 }
 
 }  // namespace
