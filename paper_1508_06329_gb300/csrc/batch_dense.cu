@@ -125,7 +125,7 @@ int fused_dense_plan(int n_max, int threads, FusedPlan *plan) {
         return set_error(CG_EINVAL, "fused batch path supports n <= %d (got %d)", kFusedMaxN, n_max);
     const int n = std::max(n_max, 1);
     FusedPlan p{};
-    if (threads == 0) threads = n <= 1024 ? 64 : n <= 2048 ? 128 : 256;
+    if (threads == 0) threads = n <= 256 ? 64 : n <= 2048 ? 128 : 256;
     if (threads != 64 && threads != 128 && threads != 256 && threads != 512)
         return set_error(CG_EINVAL, "fused batch path: unsupported CTA size %d", threads);
     p.threads = threads;

@@ -89,7 +89,9 @@ int lexbfs_dense_plan(int n_max, int threads_override, LexPlan *plan) {
     p.sort_cap = panel_sort_cap(n, room(p.state));
     p.smem_bytes = kPanelScalarBytes + panel_state_bytes(n, p.state) + panel_sort_bytes(p.sort_cap);
     p.gstate_bytes = panel_global_bytes(n, p.state);
-    int th = n <= 1024 ? 128 : n <= 2048 ? 256 : n <= 8192 ? 512 : 1024;
+    // measured on GB300 (us): n = 1,000 208 with 256 threads, 253 with 128; n = 16,384 pair 4,350 with
+    // 512, 4,570 with 1,024, 5,790 with 256
+    int th = n <= 4096 ? 256 : 512;
     if (threads_override) th = threads_override;
     if (p.state != kStateSmem) th = 1024;
     if (th != 128 && th != 256 && th != 512 && th != 1024)

@@ -32,12 +32,12 @@
 // outside have larger ids, so equality suffices.  A panel numbers 26..32
 // vertices on chordal, dense random, sparse random and tree inputs.
 //
-// Measured on GB300 (whole test, before -> now): the pair of n = 16,384 graphs
-// at density 0.1 28.5 -> 4.7 ms (8.8 us per panel of 31), G(10,000, 0.5)
-// 49.7 -> 2.5 ms, n = 41,003 104.7 -> 33.5 ms, 4,096 graphs of 16..2,048
-// vertices 3.77 -> 1.53 ms, one graph of 1,000 vertices 919 -> 244 us.  What
-// bounds a panel is latency: the rows' L2 loads, the transpose's issue slots
-// and three CTA barriers.
+// Measured on GB300 (whole test; one step per vertex -> this): the pair of
+// n = 16,384 graphs at density 0.1 28.5 -> 4.36 ms (8.2 us per panel of 31),
+// G(10,000, 0.5) 49.7 -> 1.94 ms, n = 41,003 104.7 -> 34 ms, 4,096 graphs of
+// 16..2,048 vertices 3.77 -> 1.55 ms, one graph of 1,000 vertices 919 -> 193 us.
+// What bounds a panel is latency: the rows' L2 loads, the transpose's issue
+// slots, three CTA barriers and instruction fetch.
 //
 // State: perm[] holds the vertices by position (numbered ones in front, then
 // class after class, ascending ids inside a class), and the class boundaries
@@ -95,6 +95,7 @@ struct PanelScalars {
 constexpr size_t kPanelScalarBytes = (sizeof(PanelScalars) + 15) & ~size_t(15);
 
 constexpr int kPanelWordArrays = 9;
+constexpr int kPanelCount = 1024;   // moved members of one class sorted by counting up to this many
 constexpr int kPanelFew = 16;   // pivots below which a panel is worth extending by slower rules
 constexpr int kSortCapMax = 4096;
 
@@ -397,6 +398,12 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
     using Id = typename PanelId<STATE>::type;
     constexpr int NW = T / 32;
     constexpr unsigned kAll = 0xFFFFFFFFu;
+    // Neighbouring positions per thread when split classes are rewritten: one for
+    // small CTAs (small graphs: little to do, so a short chain per position), a
+    // byte of the masks for large ones.  Both are rolled loops: code that runs
+    // once per panel is bound by instruction fetch, and the same passes unrolled
+    // eight times took 4,096 small graphs from 1.5 to 2.5 ms.
+    constexpr int G = T >= 512 ? 8 : 1;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int wn = (n + 31) >> 5;
 
@@ -422,6 +429,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
         int cp = -1;   // warp 0: the classes' last adjacent pivots, requested early
         if (warp == 0 && ppos && lane < w2) cp = __ldcg(ppos + i + lane);
         if (eb > 0) panel_write_mask<T>(emask, eb, n, st.numbered);
+        const uint32_t row_at = (uint32_t)vk * (uint32_t)stride;
         // ---- keys: a word of vertices per thread and pass
         for (int wb = warp * 32; wb < wn; wb += T) {
             const int w = wb + lane;
@@ -430,8 +438,8 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
             uint32_t r[32];
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
-                const int vj = __shfl_sync(kAll, vk, j);
-                r[j] = on && j < w2 ? rows[(size_t)vj * stride + w] : 0u;
+                const uint32_t at = __shfl_sync(kAll, row_at, j) + (uint32_t)w;   // n * stride < 2^32 words
+                r[j] = on && j < w2 ? rows[at] : 0u;
             }
             transpose32(r);
             if (on) {
@@ -680,15 +688,26 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 return b ? (q & ~31) + __ffs(b) - 1 : (q >> 5) + 1 < wn ? st.next[(q >> 5) + 1] : n;
             };
             // ---- moved members listed, the others shifted to the end of their class
-            for (int w = pw + warp; w < wn; w += NW) {
-                const uint32_t f = st.flag[w];
+            for (int q0 = (i2 & ~(G - 1)) + G * t; q0 < n; q0 += G * T) {
+                const int w = q0 >> 5, sh = q0 & 31;
+                uint32_t f = (st.flag[w] >> sh) & low_bits(min(G, n - q0));
                 if (!f) continue;
-                const int q = (w << 5) + lane;
-                if (!((f >> lane) & 1u) || q >= n) continue;
-                const Id v = st.perm[q];
-                const int s = class_start(q), e = class_end(q);
-                const int before = moved_before(q), ms = moved_before(s), me = moved_before(e);
-                if ((st.nz[w] >> lane) & 1u) {
+                const uint32_t nzw = st.nz[w] >> sh, b = st.start[w] >> sh;
+                int before = st.nzpre[w] + __popc(st.nz[w] & lanes_below(sh));
+                int s = -1, ms = 0, me = 0;   // the class at hand: its start, moved members before and up to its end
+#pragma unroll 1
+                for (; f; f &= f - 1u) {
+                    const int e = __ffs(f) - 1, q = q0 + e;
+                    if (s < 0 || ((b >> e) & 1u)) {
+                        s = class_start(q);
+                        ms = moved_before(s);
+                        me = moved_before(class_end(q));
+                    }
+                    const Id v = st.perm[q];
+                    if (!((nzw >> e) & 1u)) {
+                        st.tmp[q + me - before] = v;
+                        continue;
+                    }
                     if (r == 1) {
                         st.tmp[s + before - ms] = v;
                     } else {
@@ -697,20 +716,23 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                         st.lv[before] = v;
                         if (before == ms) atomicMax(&sc->nz_max, me - ms);
                     }
-                } else {
-                    st.tmp[q + me - before] = v;
+                    ++before;
                 }
             }
             __syncthreads();
             // ---- the moved members in their new order
             if (r > 1) {
-                if (sc->nz_max <= 64) {   // few per class: every member counts those before it
-                    for (int e = t; e < m; e += T) {
+                if (sc->nz_max <= kPanelCount) {   // four lanes count the members of e's class before e
+                    for (int e0 = warp * 8; e0 < m; e0 += NW * 8) {
+                        const int e = min(e0 + (lane >> 2), m - 1);
                         const unsigned long long c = st.comp[e];
                         const int s = (int)(c >> 44), lo = moved_before(s), hi = moved_before(class_end(s));
                         int rank = 0;
-                        for (int k = lo; k < hi; ++k) rank += st.comp[k] < c ? 1 : 0;
-                        st.tmp[s + rank] = (Id)st.lv[e];
+#pragma unroll 4
+                        for (int k = lo + (lane & 3); k < hi; k += 4) rank += st.comp[k] < c ? 1 : 0;
+                        rank += __shfl_xor_sync(kAll, rank, 1);
+                        rank += __shfl_xor_sync(kAll, rank, 2);
+                        if ((lane & 3) == 0) st.tmp[s + rank] = (Id)st.lv[e];
                     }
                 } else {
                     int p = 64;
@@ -726,31 +748,36 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 }
                 __syncthreads();
             }
-            // ---- back into perm, with the new boundaries
-            for (int w = pw + warp; w < wn; w += NW) {
-                const uint32_t f = st.flag[w];
-                if (!f) continue;
-                const int q = (w << 5) + lane;
-                const bool on = ((f >> lane) & 1u) && q < n;
-                const uint32_t b = st.start[w];
-                uint32_t k = 0u;
-                if (on) {
+            // ---- back into perm, with the new boundaries (a warp's lanes share words: old ones are read first)
+            for (int c = (i2 & ~(32 * G - 1)) + warp * 32 * G; c < n; c += T * G) {
+                const int q0 = c + G * lane, w = q0 >> 5, sh = q0 & 31;
+                uint32_t f = q0 < n ? (st.flag[w] >> sh) & low_bits(min(G, n - q0)) : 0u;
+                const uint32_t bw = q0 < n ? st.start[w] : 0u;
+                uint32_t fresh = 0u, kp = 0u;
+                if (f & ~(bw >> sh) & 1u) kp = st.key[key_slot(st.tmp[q0 - 1])] & pm;
+#pragma unroll 1
+                for (; f; f &= f - 1u) {
+                    const int e = __ffs(f) - 1, q = q0 + e;
                     const Id v = st.tmp[q];
                     st.perm[q] = v;
-                    k = st.key[key_slot(v)] & pm;
+                    const uint32_t k = st.key[key_slot(v)] & pm;
+                    if (k != kp && !((bw >> (sh + e)) & 1u)) {
+                        fresh |= 1u << e;
+                        // the members that did not move keep the class's last adjacent pivot
+                        if (ppos && k == 0u) {
+                            const uint32_t le = bw & low_bits(sh + e + 1);
+                            ppos[q] = __ldcg(ppos + (le ? (w << 5) + 31 - __clz(le) : st.last[w - 1]));
+                        }
+                    }
+                    kp = k;
                 }
-                uint32_t kp = __shfl_up_sync(kAll, k, 1);
-                const bool inside = on && !((b >> lane) & 1u);
-                if (lane == 0 && inside) kp = st.key[key_slot(st.tmp[q - 1])] & pm;
-                const bool fresh = inside && k != kp;
-                const uint32_t nb = __ballot_sync(kAll, fresh);
-                // the members that did not move keep the class's last adjacent pivot
-                if (ppos && fresh && k == 0u) {
-                    const uint32_t le = b & low_bits(lane + 1);
-                    ppos[q] = __ldcg(ppos + (le ? (w << 5) + 31 - __clz(le) : st.last[w - 1]));
+                if constexpr (G == 1) {
+                    const uint32_t nb = __ballot_sync(kAll, fresh != 0u);
+                    if (lane == 0 && nb) st.start[w] = bw | nb;
+                } else {
+                    __syncwarp();
+                    if (fresh) reinterpret_cast<uint8_t *>(&st.start[w])[sh >> 3] = (uint8_t)((bw >> sh) | fresh);
                 }
-                __syncwarp();
-                if (lane == 0 && nb) st.start[w] = b | nb;
             }
             __syncthreads();
             break;
@@ -767,14 +794,23 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
             if (eb == 0 || i + lane < 32 * eb) atomicOr(&st.numbered[v >> 5], 1u << (v & 31));
         }
         if (ppos) {
-            for (int q0 = (i2 & ~7) + 8 * t; q0 < n; q0 += 8 * T) {
-                uint32_t b = reinterpret_cast<const uint8_t *>(&st.start[q0 >> 5])[(q0 >> 3) & 3];
-                if (q0 < i2) b &= 0xFFu << (i2 - q0);
-                for (; b; b &= b - 1u) {
-                    const int q = q0 + __ffs(b) - 1;
-                    const uint32_t k = st.key[key_slot(st.perm[q])] & pm;
-                    if (k) ppos[q] = sc->piv[32 - __ffs(pivot_key(k))];
+            constexpr int U = 4;   // words at once, so that their gathers overlap
+            for (int w0 = (i2 >> 5) + warp; w0 < wn; w0 += U * NW) {
+                Id v[U];
+                uint32_t k[U];
+                bool on[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int w = min(w0 + u * NW, wn - 1), q = (w << 5) + lane;
+                    on[u] = w == w0 + u * NW && q >= i2 && q < n && ((st.start[w] >> lane) & 1u);
+                    v[u] = st.perm[q];
                 }
+#pragma unroll
+                for (int u = 0; u < U; ++u) k[u] = on[u] ? st.key[key_slot(v[u])] & pm : 0u;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (k[u])
+                        ppos[((w0 + u * NW) << 5) + lane] = sc->piv[ident ? 31 - __clz(k[u]) : 32 - __ffs(pivot_key(k[u]))];
             }
         }
         i = i2;
