@@ -103,7 +103,7 @@ __device__ __forceinline__ void prefetch_range_l2(const void *base, size_t bytes
 // CG_ECUDA with a description (CG_DEBUG_CHECK).
 #ifdef CG_BOUNDS_CHECK
 static __device__ unsigned long long cg_dbg_word;       // this translation unit's error word
-static __device__ unsigned long long cg_dbg_sink[2];    // target of redirected accesses
+static __device__ __align__(16) unsigned long long cg_dbg_sink[2];    // target of redirected accesses
 
 __device__ __forceinline__ void cg_dbg_record(unsigned code, unsigned long long idx) {
     atomicCAS(&cg_dbg_word, 0ull, ((unsigned long long)(code & 0xFFu) << 56) | (idx & ((1ull << 56) - 1)));
@@ -139,9 +139,7 @@ __device__ __forceinline__ T *cg_arr(T *p, unsigned long long, unsigned) {
 // Array codes of the bounds-checking build (the high byte of the error word).
 enum : unsigned {
     kChkCls = 1, kChkPerm, kChkKey, kChkSplit, kChkSort, kChkNumbered,
-    kChkCsrCls = 16, kChkCsrVnext, kChkCsrVprev, kChkCsrCnext, kChkCsrCprev, kChkCsrCfirst, kChkCsrClast,
-    kChkCsrCsize, kChkCsrCmoved, kChkCsrCchild, kChkCsrFree, kChkCsrSy, kChkCsrSop, kChkCsrSon, kChkCsrSrun,
-    kChkCsrSkey,
+    kChkCsrCls = 16, kChkCsrNext, kChkCsrRec, kChkCsrFree, kChkCsrSub, kChkCsrSkey, kChkCsrArena,
     kChkUnitMask = 40, kChkUnitPos, kChkUnitRow, kChkUnitGroup,
     kChkInjected = 255,
 };
