@@ -33,21 +33,12 @@ const char *cg_debug_array_name(unsigned code) {
         case kChkSort: return "dense LexBFS split sort";
         case kChkNumbered: return "dense LexBFS numbered mask";
         case kChkCsrCls: return "CSR LexBFS cls";
-        case kChkCsrVnext: return "CSR LexBFS vnext";
-        case kChkCsrVprev: return "CSR LexBFS vprev";
-        case kChkCsrCnext: return "CSR LexBFS class next";
-        case kChkCsrCprev: return "CSR LexBFS class prev";
-        case kChkCsrCfirst: return "CSR LexBFS class first";
-        case kChkCsrClast: return "CSR LexBFS class last";
-        case kChkCsrCsize: return "CSR LexBFS class size";
-        case kChkCsrCmoved: return "CSR LexBFS class moved";
-        case kChkCsrCchild: return "CSR LexBFS class child";
+        case kChkCsrNext: return "CSR LexBFS class next";
+        case kChkCsrRec: return "CSR LexBFS class record";
         case kChkCsrFree: return "CSR LexBFS free stack";
-        case kChkCsrSy: return "CSR LexBFS long-row vertices";
-        case kChkCsrSop: return "CSR LexBFS long-row old prev";
-        case kChkCsrSon: return "CSR LexBFS long-row old next";
-        case kChkCsrSrun: return "CSR LexBFS long-row runs";
+        case kChkCsrSub: return "CSR LexBFS long-row classes";
         case kChkCsrSkey: return "CSR LexBFS long-row keys";
+        case kChkCsrArena: return "CSR LexBFS arena";
         case kChkUnitMask: return "check earlier-than mask";
         case kChkUnitPos: return "check pos gather";
         case kChkUnitGroup: return "check order / parent value";
@@ -778,7 +769,6 @@ int run_mcs_dense(cg_context *ctx, const cg_dense *g, int32_t *order_out, int32_
     const size_t o_pos = cv.take<int32_t>(n);
     const size_t o_parent = cv.take<int32_t>(n);
     const size_t o_key = cv.take<unsigned long long>(2);
-    const size_t o_counter = cv.take<int>(1);
     const size_t o_emask = cv.take<uint32_t>(res ? earlier_mask_words(n) : 0);
     int rc;
     if ((rc = ensure_ws(ctx, cv.off))) return rc;
@@ -788,7 +778,7 @@ int run_mcs_dense(cg_context *ctx, const cg_dense *g, int32_t *order_out, int32_
     const DenseDesc d = desc_of(g, 0, 0);
     if (n > 0) {
         PhaseTimer pt(ctx, &ctx->ev_lex, stream);
-        if ((rc = mcs_dense_launch(nullptr, d, 1, n, 1, order, pos, at<int>(ctx, o_counter), stream))) return rc;
+        if ((rc = mcs_dense_launch(d, order, pos, stream))) return rc;
         ctx->launches += 1;
     }
     if (!res) return CG_OK;

@@ -128,9 +128,8 @@ int sweep_csr_relabel_launch(int n, int64_t nnz, const int64_t *row_ptr, const i
 int sweep_order_launch(const DenseDesc &d, const LexPlan &plan, void *gstate, int *counter, const SweepBuffers &sb,
                        int32_t *order, int32_t *pos, int num_sms, cudaStream_t stream);
 
-// ---- dense MCS (mcs_dense.cu): one CTA per graph, n <= 65520
-int mcs_dense_launch(const DenseDesc *descs, DenseDesc single, int count, int n_max, int ctas, int32_t *order,
-                     int32_t *pos, int *work_counter, cudaStream_t stream);
+// ---- dense MCS (mcs_dense.cu): one CTA, n <= 65520
+int mcs_dense_launch(DenseDesc d, int32_t *order, int32_t *pos, cudaStream_t stream);
 
 // ---- CSR LexBFS (lexbfs_csr.cu): one CTA per graph (warp 0 walks the steps), state in `ws`
 size_t lexbfs_csr_workspace_bytes(int64_t n, int64_t max_deg);
