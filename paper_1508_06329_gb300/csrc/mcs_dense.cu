@@ -26,7 +26,7 @@
 // A panel numbers about 31 vertices on dense chordal graphs and 10 on
 // G(n, 1/2).
 //
-// The counts (16 bits; 0xFFFF: numbered, or in the window) and the keys of
+// The counts (16 bits, plus one; 0: numbered, or in the window) and the keys of
 // kMcsKeyWords words of vertices are in shared memory; a larger graph passes
 // over its rows twice per panel, in chunks.
 #include <algorithm>
@@ -43,11 +43,10 @@ constexpr int kMcsWorkers = 512;                // threads that hold vertices
 constexpr int kMcsThreads = kMcsWorkers + 32;   // and the warp that visits the window
 constexpr int kMcsGroups = 128;
 constexpr int kMcsCand = 512;
-constexpr unsigned kMcsNone = 0xFFFFu;
 constexpr size_t kMcsSmem = 220 * 1024;
 
 struct McsShared {
-    const uint32_t *row[32];      // the window's rows
+    uint4 row4[8];                // four times the window's vertices
     int v[32];                    // the window, largest (count, id) first
     int cnt[32];
     uint32_t mask[33];            // window vertices among the first j pivots
@@ -78,11 +77,11 @@ __global__ void __launch_bounds__(kMcsThreads, 1) mcs_dense_kernel(DenseDesc d, 
     uint32_t *key = reinterpret_cast<uint32_t *>(smem);                     // [32 * key_words]
     uint16_t *cnt = reinterpret_cast<uint16_t *>(smem + (size_t)key_words * 128);   // [32 * wn]
     prefetch_range_l2<kMcsThreads>(rows, (size_t)n * d.words * sizeof(uint32_t));
-    for (int v = t; v < 32 * wn; v += kMcsThreads) cnt[v] = v < n ? 0 : kMcsNone;
+    for (int v = t; v < 32 * wn; v += kMcsThreads) cnt[v] = v < n ? 1 : 0;
     if (t < 32) {
         sh.v[t] = t;
-        sh.cnt[t] = 0;
-        sh.row[t] = rows + (size_t)min(t, n - 1) * d.words;
+        sh.cnt[t] = 1;
+        reinterpret_cast<unsigned *>(sh.row4)[t] = 4u * min(t, n - 1);
     }
     __syncthreads();
 
@@ -97,8 +96,7 @@ __global__ void __launch_bounds__(kMcsThreads, 1) mcs_dense_kernel(DenseDesc d, 
             for (int wb = warp * 32; wb < we; wb += kMcsWorkers) {
                 const int w = wb + lane;
                 uint32_t r[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) r[j] = w < we && j < w2 ? __ldg(sh.row[j] + w0 + w) : 0u;
+                panel_load_rows(rows + min(w0 + w, wn - 1), d.words, sh.row4, r);   // (key bits from w2 on: not read)
                 transpose32(r);
                 if (w < we) {
 #pragma unroll
@@ -125,12 +123,11 @@ __global__ void __launch_bounds__(kMcsThreads, 1) mcs_dense_kernel(DenseDesc d, 
             myv = lane < w2 ? sh.v[lane] : 0;
             mycnt = sh.cnt[lane];
             uint32_t a[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) a[j] = j < w2 ? __ldg(sh.row[j] + (myv >> 5)) : 0u;
+            panel_load_rows(rows + (myv >> 5), d.words, sh.row4, a);
 #pragma unroll
             for (int j = 0; j < 32; ++j) adj |= ((a[j] >> (myv & 31)) & 1u) << j;
             adj &= ~(1u << lane);
-            if (lane < w2) cnt[myv] = kMcsNone;
+            if (lane < w2) cnt[myv] = 0;
             unsigned comp = lane < w2 ? mcs_comp(mycnt, myv) : 0u;
             uint32_t done = 0u, m8 = 0u;
             unsigned b8 = kAll;
@@ -176,6 +173,8 @@ __global__ void __launch_bounds__(kMcsThreads, 1) mcs_dense_kernel(DenseDesc d, 
         unsigned b8[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) m8[k] = sh.mask8[k], b8[k] = sh.beat8[k];
+        const int least = (int)(min(min(b8[0], b8[1]), min(b8[2], b8[3])) >> 16);
+        const unsigned near = max(least - 32, 1);
         int r = w2;
         for (int ch = 0; ch < chunks; ++ch) {
             const int w0 = ch * key_words;
@@ -188,24 +187,23 @@ __global__ void __launch_bounds__(kMcsThreads, 1) mcs_dense_kernel(DenseDesc d, 
                 const int qe = 4 * min(key_words, wn - w0);
                 for (int q = t; q < qe; q += kMcsWorkers) {
                     uint16_t c[8];
-                    uint32_t k[8];
-                    load8(w0, q, c, k);
+                    panel_load8(cnt + 32 * w0 + 8 * q, c);
                     const unsigned v0 = 32 * w0 + 8 * q;
-                    uint32_t in = 0u;
+                    uint32_t in = 0u;   // within 32 of the least beat
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        bool over = false;
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) over |= mcs_comp(c[e] + __popc(k[e] & m8[b]), v0 + e) > b8[b];
-                        in |= (over && c[e] != kMcsNone ? 1u : 0u) << e;
-                    }
+                    for (int e = 0; e < 8; ++e) in |= (c[e] >= near ? 1u : 0u) << e;
+#pragma unroll 1
                     for (; in; in &= in - 1u) {
                         const int e = __ffs(in) - 1;
                         const unsigned ce = cnt[v0 + e];
                         const int w = q >> 2, p = ((q & 3) << 1) + (e >> 2);
                         const uint32_t ke = key[32 * w + ((p ^ (w & 7)) << 2) + (e & 3)];
-                        for (int j = 0; j < r; ++j)
-                            if (mcs_comp(ce + __popc(ke & sh.mask[j]), v0 + e) > sh.beat[j]) r = j;
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            if (mcs_comp(ce + __popc(ke & m8[b]), v0 + e) <= b8[b]) continue;
+                            for (int j = 8 * b; j < min(8 * b + 8, r); ++j)
+                                if (mcs_comp(ce + __popc(ke & sh.mask[j]), v0 + e) > sh.beat[j]) r = j;
+                        }
                     }
                 }
             }
@@ -247,7 +245,7 @@ __global__ void __launch_bounds__(kMcsThreads, 1) mcs_dense_kernel(DenseDesc d, 
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     unsigned ce = c[e];
-                    if (ce != kMcsNone) {
+                    if (ce) {
                         ce += __popc(k[e] & taken);
                         best[e] = max(best[e], mcs_comp(ce, v0 + e));
                     }
@@ -290,7 +288,7 @@ __global__ void __launch_bounds__(kMcsThreads, 1) mcs_dense_kernel(DenseDesc d, 
                     uint32_t in = 0u;
 #pragma unroll
                     for (int e = 0; e < 8; ++e)
-                        in |= (c[e] != kMcsNone && mcs_comp(c[e], 8 * q + e) >= bound ? 1u : 0u) << e;
+                        in |= (c[e] && mcs_comp(c[e], 8 * q + e) >= bound ? 1u : 0u) << e;
                     if (in) {
                         int at = atomicAdd(&sh.ncand, __popc(in));
                         for (; in; in &= in - 1u) {
@@ -323,7 +321,7 @@ __global__ void __launch_bounds__(kMcsThreads, 1) mcs_dense_kernel(DenseDesc d, 
                 const int v = 65535 - (int)(mine & 0xFFFFu);
                 sh.v[rank] = v;
                 sh.cnt[rank] = (int)(mine >> 16);
-                sh.row[rank] = rows + (size_t)v * d.words;
+                reinterpret_cast<unsigned *>(sh.row4)[rank] = 4u * v;
             }
         }
         __syncthreads();
