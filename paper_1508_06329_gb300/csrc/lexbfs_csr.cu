@@ -29,13 +29,20 @@
 // is never stored: its members are the v with cls[v] = n, in id order.
 // The first classes of the list are taken out of it ahead of time into the
 // front, an array of up to 128 vertices in partition order in shared memory
-// (warp 0 does that while the other warps gather the window's rows); classes in
-// the front are split there.  A class too large for the front is entered 32
+// (warp 0 does that while the other warps, the workers, gather, order and sort);
+// classes in the front are split there.  A class too large for the front is entered 32
 // members at a time; what a panel leaves of those goes back.
 // Rows longer than the hash table takes (kMaxEntries) make a panel of one
-// pivot, whose neighbours are sorted by (class, row position) in the workspace.
+// pivot, whose neighbours are sorted by (class, row position) in the workspace;
+// those without a numbered neighbour need no sort.
 // parent[y]: the last pivot of the last panel that met y, p(y) of the
 // perfect-elimination check (Section 5.2).
+//
+// Measured on GB300 (whole test, one step per vertex -> panels): 65,536 vertices
+// of degree 21 122.3 -> 26.4 ms, 262,143 515 -> 126 ms, 5,000 8.0 -> 2.8 ms, 20,000
+// of degree 5 28.0 -> 8.6 ms.  A panel of 30 pivots takes about 12 us: gathering
+// 2, the order 1.7, sorting 3, new classes 4.5, the front and barriers the rest;
+// all of it latency (barriers, dependent loads from L2, instruction fetch).
 #include <algorithm>
 
 #include "kernels.h"
@@ -51,9 +58,11 @@ constexpr int kHead = -4;              // predecessor of the first class
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
 constexpr int kCsrArrays = 11;         // the state's size in blocks of n + 1 ints, without the long rows' arrays
+// 65,536 / 5,000 vertices of degree 21: 26.4 / 2.8 ms with 1,024 threads, 27.9 / 3.6 with 512, 33.8 / 5.5 with 256
 constexpr int kCsrThreads = 1024;
+constexpr int kCsrWorkers = kCsrThreads - 32;   // all but warp 0, which fills the front
 constexpr int kMaxEntries = 2048;      // row entries of one panel
-constexpr int kHashSize = 4096;        // at least kMaxEntries + 2 kFrontCap
+constexpr int kHashSize = 4096;        // at least kMaxEntries + kFrontCap
 constexpr int kFrontCap = 128;
 constexpr int kFrontLow = 64;          // the front is filled up to this many vertices beyond the window
 constexpr int kNextSmem = 30 * 1024;   // next pointers kept in shared memory
@@ -73,6 +82,7 @@ struct CsrState {
 
 __host__ __device__ inline int64_t pow2_at_least(int64_t x) {
     int64_t p = 1;
+#pragma unroll 1
     while (p < x) p <<= 1;
     return p;
 }
@@ -110,14 +120,16 @@ struct Front {                         // vertices in partition order
 };
 
 struct CsrShared {
+    // (a long row's digit counts lie in the first two arrays)
     unsigned long long key[kMaxEntries];    // moved vertices: class << 32 | inverted label
     unsigned long long key2[kMaxEntries];   // listed: class << 32 | hash slot; then moved, sorted
+    int hkey[kHashSize];                    // vertex (-1: free)
+    uint32_t hmask[kHashSize];              // its key
     int y[kMaxEntries];
     int y2[kMaxEntries];
     int sub[kMaxEntries];                   // new class by sorted index
-    int hkey[kHashSize];                    // vertex (-1: free)
-    uint32_t hmask[kHashSize];              // its key
-    uint8_t hfront[kHashSize];              // it came to the front in this panel
+    uint32_t gstart[kMaxEntries / 32];      // bit k: the sorted index k is the first of its new class
+    uint32_t cstart[kMaxEntries / 32];      // and of its old class
     Front front[2];
     int fslot[kFrontCap];                   // hash slot
     unsigned fat[kFrontCap];                // slot in the arena (large class in the front)
@@ -139,11 +151,13 @@ struct CsrShared {
     uint32_t bit[32];
     uint32_t tab[8][16];
     int scan[32];
+    int unl_id;                             // long row: the new class of the vertices without a numbered neighbour
     int next[1];                            // [next_smem]
 };
 
 __global__ void csr_init_kernel(int *ws, int64_t n, int64_t max_deg, int32_t *parent) {
     CsrState s = csr_state_carve(ws, n, max_deg);
+#pragma unroll 1
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         s.cls[v] = (int)n;
         s.freel[v] = (int)(n - 1 - v);   // taken from the end: low ids first
@@ -152,49 +166,75 @@ __global__ void csr_init_kernel(int *ws, int64_t n, int64_t max_deg, int32_t *pa
     }
 }
 
-// Sorts key[0..p), p > tile_n a power of two, in global memory (bitonic, all
-// threads of the CTA): the passes with a stride below tile_n pair keys inside one aligned tile of tile_n keys, so they
-// run on a shared-memory copy of each tile (the first log2 of them for every k
-// up to the tile size, the rest after each k's global passes).
-__device__ void cta_sort_keys_tiled(unsigned long long *key, int64_t p, unsigned long long *tile, int tile_n) {
-    const int T = blockDim.x;
-    auto tile_passes = [&](int64_t t0, int64_t k_lo, int64_t k_hi, int64_t j_first) {
-        for (int li = threadIdx.x; li < tile_n; li += T) tile[li] = key[t0 + li];
-        __syncthreads();
-        for (int64_t k = k_lo; k <= k_hi; k <<= 1) {
-            for (int64_t j = (k == k_lo ? j_first : (k >> 1)); j > 0; j >>= 1) {
-                for (int li = threadIdx.x; li < tile_n; li += T) {
-                    const int l = li ^ (int)j;
-                    if (l > li) {
-                        const unsigned long long a = tile[li], b = tile[l];
-                        if ((a > b) == (((t0 + li) & k) == 0)) {
-                            tile[li] = b;
-                            tile[l] = a;
-                        }
-                    }
-                }
-                __syncthreads();
-            }
-        }
-        for (int li = threadIdx.x; li < tile_n; li += T) key[t0 + li] = tile[li];
-        __syncthreads();
-    };
-    for (int64_t t0 = 0; t0 < p; t0 += tile_n) tile_passes(t0, 2, tile_n, 1);   // k = 2 .. tile size
-    for (int64_t k = 2 * (int64_t)tile_n; k <= p; k <<= 1) {
-        for (int64_t j = k >> 1; j >= tile_n; j >>= 1) {
-            for (int64_t i = threadIdx.x; i < p; i += T) {
-                const int64_t l = i ^ j;
-                if (l > i) {
-                    const unsigned long long a = key[i], b = key[l];
-                    if ((a > b) == ((i & k) == 0)) {
-                        key[i] = b;
-                        key[l] = a;
-                    }
+// A barrier of some of the CTA's warps.
+__device__ __forceinline__ void named_barrier(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Sorts the moved vertices key/y[0..m) by (key, y) into key2/y2, m <= kMaxEntries:
+// every warp sorts 32 in registers, then a vertex's rank is its place in its run
+// plus the vertices before it in every other run, found by bisection, two runs
+// at a time.  (About 300 are moved on the sparse chordal graphs: 15,000 cycles by
+// comparing all with all.)  One barrier of the workers; the caller has the ones
+// around.
+__device__ void panel_sort_moved(CsrShared *sh, int m) {
+    constexpr int T = kCsrWorkers;
+    const int t = threadIdx.x - 32, lane = t & 31, warp = warp_index() - 1;
+    const int runs = (m + 31) >> 5;
+#pragma unroll 1
+    for (int b = warp; b < runs; b += T / 32) {
+        const int e = 32 * b + lane;
+        unsigned long long k = e < m ? sh->key[e] : ~0ull;
+        int y = e < m ? sh->y[e] : 0x7FFFFFFF;
+#pragma unroll 1
+        for (int s = 2; s <= 32; s <<= 1)
+#pragma unroll 1
+            for (int j = s >> 1; j > 0; j >>= 1) {
+                const unsigned long long ok = __shfl_xor_sync(kFull, k, j);
+                const int oy = __shfl_xor_sync(kFull, y, j);
+                const bool greater = k > ok || (k == ok && y > oy);
+                if (greater == (((lane & s) == 0) == ((lane & j) == 0))) {
+                    k = ok;
+                    y = oy;
                 }
             }
-            __syncthreads();
+        sh->key[e] = k;
+        sh->y[e] = y;
+    }
+    named_barrier(1, kCsrWorkers);
+    int lg = 4;   // lanes per vertex
+    while (lg > 0 && (32 * runs << lg) > T) --lg;
+    const int step = 1 << lg;
+#pragma unroll 1
+    for (int e = t >> lg; e < 32 * runs; e += T) {   // whole warps: a warp's elements are of one run
+        const unsigned long long k = sh->key[e];
+        const int y = sh->y[e], own = e >> 5;
+        int rank = 0;
+#pragma unroll 1
+        for (int b0 = t & (step - 1); b0 < runs; b0 += 2 * step) {
+            int lo[2] = {0, 0};
+            auto before = [&](int b, int i) {   // element i of run b is before this one
+                const unsigned long long x = sh->key[32 * b + i];
+                return x < k || (x == k && sh->y[32 * b + i] < y);
+            };
+#pragma unroll
+            for (int st = 16; st > 0; st >>= 1)
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (before(min(b0 + u * step, runs - 1), lo[u] + st - 1)) lo[u] += st;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int b = b0 + u * step;
+                if (b < runs && b != own) rank += lo[u] + (before(b, lo[u]) ? 1 : 0);
+            }
         }
-        for (int64_t t0 = 0; t0 < p; t0 += tile_n) tile_passes(t0, k, k, tile_n >> 1);
+#pragma unroll 1
+        for (int o = 1; o < step; o <<= 1) rank += __shfl_xor_sync(kFull, rank, o);
+        rank += e & 31;
+        if ((t & (step - 1)) == 0 && rank < m) {
+            sh->key2[rank] = k;
+            sh->y2[rank] = y;
+        }
     }
 }
 
@@ -216,10 +256,11 @@ __device__ __forceinline__ void set_next(const CsrState &s, CsrShared *sh, const
 }
 
 // y's slot of the hash table, taken if it was not there.  At most kMaxEntries +
-// 2 kFrontCap vertices meet the table's kHashSize slots, so a free one is found.
+// kFrontCap vertices meet the table's kHashSize slots, so a free one is found.
 __device__ __forceinline__ int hash_slot(CsrShared *sh, int y, bool *fresh) {
     unsigned h = ((unsigned)y * 2654435761u) >> 20;   // 12 bits: kHashSize
     *fresh = false;
+#pragma unroll 1
     for (int k = 0; k < kHashSize; ++k) {
         const int old = atomicCAS(&sh->hkey[h], -1, y);
         if (old == -1) *fresh = true;
@@ -227,6 +268,19 @@ __device__ __forceinline__ int hash_slot(CsrShared *sh, int y, bool *fresh) {
         h = (h + 1) & (kHashSize - 1);
     }
     return (int)h;
+}
+
+// y's key, 0 when it is not in the table.
+__device__ __forceinline__ uint32_t hash_key(const CsrShared *sh, int y) {
+    unsigned h = ((unsigned)y * 2654435761u) >> 20;
+#pragma unroll 1
+    for (int k = 0; k < kHashSize; ++k) {
+        const int x = sh->hkey[h];
+        if (x == y) return sh->hmask[h];
+        if (x == -1) break;
+        h = (h + 1) & (kHashSize - 1);
+    }
+    return 0u;
 }
 
 __device__ __forceinline__ int warp_inclusive(int v) {
@@ -249,9 +303,84 @@ __device__ __forceinline__ int warp_owner(unsigned incl, unsigned e) {
     return p;
 }
 
-// Puts v at position p of the front.
-__device__ __forceinline__ void front_put(CsrShared *sh, Front *f, const CsrGraph &g, int p, int v, int par) {
-    const int64_t b = g.row_ptr[v], e = g.row_ptr[v + 1];
+// A long row's vertices in the order of (class, row position): kept[k] is the
+// class of the row's k-th vertex (-1: none of them), m how many there are.  A
+// radix sort by class, eight bits a pass, each warp over its own part of the
+// row, between the buffers b1 and b2; returns the one with the result, keys
+// (class << 32 | row position).  (25,000 vertices: 15,000 cycles; a bitonic
+// network on 8,192 keys at a time in shared memory took 500,000.)
+__device__ const unsigned long long *sort_long_row(CsrShared *sh, const int *kept, int d, int m, int n,
+                                                   unsigned long long *b1, unsigned long long *b2) {
+    constexpr int NW = kCsrThreads / 32;
+    const int t = threadIdx.x, lane = t & 31, warp = warp_index();
+    uint32_t(*hist)[256] = reinterpret_cast<uint32_t(*)[256]>(sh->key);   // [NW][256]: key and key2
+    unsigned long long *src = b2, *dst = b1;
+#pragma unroll 1
+    for (int shift = 0; shift == 0 || ((n - 1) >> shift) > 0; shift += 8) {
+        const int len = shift ? m : d, part = (len + kCsrThreads - 1) / kCsrThreads * 32;
+        const int lo = min(warp * part, len), hi = min(lo + part, len);
+        auto load = [&](int k) -> unsigned long long {   // ~0: none
+            if (k >= hi) return ~0ull;
+            if (shift) return src[k];
+            const int c = kept[k];
+            return c < 0 ? ~0ull : (unsigned long long)(unsigned)c << 32 | (unsigned)k;
+        };
+        auto digit = [&](unsigned long long x) -> unsigned {
+            return x == ~0ull ? 256u : (unsigned)(x >> (32 + shift)) & 255u;
+        };
+        for (int k = t; k < NW * 256; k += kCsrThreads) hist[k >> 8][k & 255] = 0u;
+        __syncthreads();
+        unsigned long long ahead = load(lo + lane);
+#pragma unroll 1
+        for (int k0 = lo; k0 < hi; k0 += 32) {
+            const unsigned g = digit(ahead);
+            ahead = load(k0 + 32 + lane);
+            const uint32_t same = __match_any_sync(kFull, g);
+            if (g < 256u && (same & lanes_below(lane)) == 0u) hist[warp][g] += __popc(same);
+            __syncwarp();
+        }
+        __syncthreads();
+        // where each warp's share of each digit begins: thread t sums warps [w0, w0 + PER) of one digit
+        constexpr int PER = NW * 256 / kCsrThreads;
+        const int g = t / (NW / PER), w0 = t % (NW / PER) * PER;
+        int mine = 0;
+        for (int w = 0; w < PER; ++w) mine += hist[w0 + w][g];
+        const int incl = warp_inclusive(mine);
+        if (lane == 31) sh->scan[warp] = incl;
+        __syncthreads();
+        const int wc = lane < NW ? sh->scan[lane] : 0;
+        int at = __reduce_add_sync(kFull, lane < warp ? wc : 0) + incl - mine;
+        for (int w = 0; w < PER; ++w) {
+            const int x = hist[w0 + w][g];
+            hist[w0 + w][g] = at;
+            at += x;
+        }
+        __syncthreads();
+        ahead = load(lo + lane);
+#pragma unroll 1
+        for (int k0 = lo; k0 < hi; k0 += 32) {
+            const unsigned long long x = ahead;
+            const unsigned h = digit(x);
+            ahead = load(k0 + 32 + lane);
+            const uint32_t same = __match_any_sync(kFull, h), below = same & lanes_below(lane);
+            const uint32_t base = h < 256u ? hist[warp][h] : 0u;
+            __syncwarp();
+            if (h < 256u) {
+                dst[base + __popc(below)] = x;
+                if (below == 0u) hist[warp][h] = base + __popc(same);
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+        unsigned long long *const u = src;
+        src = dst;
+        dst = u;
+    }
+    return src;
+}
+
+// Puts v, whose row is col[b, e), at position p of the front.
+__device__ __forceinline__ void front_put(Front *f, int p, int v, int par, int64_t b, int64_t e) {
     f->v[p] = v;
     f->par[p] = par;
     f->beg[p] = b;
@@ -271,6 +400,7 @@ __device__ void front_fill(const CsrState &s, CsrShared *sh, const CsrGraph &g, 
         // the next classes' ids: lane k the k-th
         int id = top, mine = g.n, cnt = 0, after = g.n;
         const int lim = min(32, want);
+#pragma unroll 1
         for (; cnt < lim && id != g.n; ++cnt) {
             if (lane == cnt) mine = id;
             id = get_next(s, sh, g, id);
@@ -289,10 +419,11 @@ __device__ void front_fill(const CsrState &s, CsrShared *sh, const CsrGraph &g, 
                 if (lane >= o) slots += u;
             }
             const unsigned total = __shfl_sync(kFull, slots, 31);
-            constexpr int U = 2;
+            constexpr int U = 4;   // slots per lane at once, so that their loads overlap
+#pragma unroll 1
             for (unsigned b = 0; b < total; b += 32 * U) {
-                int v[U], own[U], pv[U];
-                bool live[U];
+                int v[U], own[U], c[U], pv[U];
+                int64_t rb[U], re[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const unsigned e = b + 32 * u + lane;
@@ -302,30 +433,33 @@ __device__ void front_fill(const CsrState &s, CsrShared *sh, const CsrGraph &g, 
                     v[u] = e < total ? s.arena[at] : -1;
                 }
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int c = __shfl_sync(kFull, mine, own[u]);
-                    live[u] = v[u] >= 0 && s.cls[v[u]] == c;
-                    pv[u] = live[u] && g.parent ? g.parent[v[u]] : -1;
+                for (int u = 0; u < U; ++u) {   // (also for slots whose vertex has left)
+                    const int x = max(v[u], 0);
+                    c[u] = v[u] >= 0 ? s.cls[x] : kNumberedCls;
+                    rb[u] = g.row_ptr[x];
+                    re[u] = g.row_ptr[x + 1];
+                    pv[u] = g.parent ? g.parent[x] : -1;
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
+                    if (b + 32 * u >= total) break;
+                    const bool live = c[u] == __shfl_sync(kFull, mine, own[u]);
                     const int first = have + __shfl_sync(kFull, incl - sz, own[u]);
-                    const unsigned lm = __ballot_sync(kFull, live[u]);
+                    const unsigned lm = __ballot_sync(kFull, live);
                     const int p = len + __popc(lm & lanes_below(lane));
-                    if (live[u] && p < kFrontCap) {
-                        front_put(sh, f, g, p, v[u], pv[u]);
+                    if (live && p < kFrontCap) {
+                        front_put(f, p, v[u], pv[u], rb[u], re[u]);
                         s.cls[v[u]] = kFrontCls;
                         if (p == first) atomicOr(&sh->fstart[p >> 5], 1u << (p & 31));
-                        bool fresh;
-                        const int h = hash_slot(sh, v[u], &fresh);
-                        sh->fslot[p] = h;
-                        sh->hfront[h] = 1;
                     }
                     len = min(len + __popc(lm), kFrontCap);
                 }
             }
             const int nx = ntake < cnt ? __shfl_sync(kFull, mine, ntake) : after;
-            if (take) s.freel[sh->free_top + lane] = mine;
+            if (take) {
+                s.freel[sh->free_top + lane] = mine;
+                s.rec[mine].z = -1;   // what the panel lists of it stays in the front
+            }
             __syncwarp();
             if (lane == 0) {
                 sh->free_top += ntake;
@@ -347,6 +481,7 @@ __device__ void front_fill(const CsrState &s, CsrShared *sh, const CsrGraph &g, 
     constexpr int U = 4;
     unsigned found_at = 0u;
     const unsigned end = (unsigned)r0.y;
+#pragma unroll 1
     for (unsigned b = (unsigned)r0.x; b < end && len < 32; b += 32 * U) {
         if (len > 0 && b - found_at >= (unsigned)kScanStop) break;
         int v[U];
@@ -363,7 +498,7 @@ __device__ void front_fill(const CsrState &s, CsrShared *sh, const CsrGraph &g, 
             const unsigned lm = __ballot_sync(kFull, live[u]);
             const int p = len + __popc(lm & lanes_below(lane));
             if (live[u] && p < 32) {
-                front_put(sh, f, g, p, v[u], g.parent ? g.parent[v[u]] : -1);
+                front_put(f, p, v[u], g.parent ? g.parent[v[u]] : -1, g.row_ptr[v[u]], g.row_ptr[v[u] + 1]);
                 s.cls[v[u]] = kFrontCls;
                 sh->fat[p] = b + 32 * u + lane;
             }
@@ -384,9 +519,10 @@ __device__ void front_fill(const CsrState &s, CsrShared *sh, const CsrGraph &g, 
 
 // Packs the arena's live segments (all threads).
 __device__ void arena_pack(const CsrState &s, CsrShared *sh, const CsrGraph &g) {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, lane = t & 31, warp = warp_index();
     const unsigned top = sh->atop;
     unsigned out = 0u;
+#pragma unroll 1
     for (unsigned b = 0; b < top; b += kCsrThreads) {
         const unsigned a = b + t;
         int v = -1;
@@ -403,12 +539,13 @@ __device__ void arena_pack(const CsrState &s, CsrShared *sh, const CsrGraph &g) 
         const unsigned lm = __ballot_sync(kFull, v >= 0);
         if (lane == 0) sh->scan[warp] = __popc(lm);
         __syncthreads();   // the chunk is read before it is written
-        const int wc = sh->scan[lane];
+        const int wc = lane < kCsrThreads / 32 ? sh->scan[lane] : 0;
         const int before = __reduce_add_sync(kFull, lane < warp ? wc : 0), all = __reduce_add_sync(kFull, wc);
         if (v >= 0) s.arena[out + before + __popc(lm & lanes_below(lane))] = v;
         out += all;
         __syncthreads();
     }
+#pragma unroll 1
     for (unsigned a = t; a < out; a += kCsrThreads) {
         const int c = s.cls[s.arena[a]];
         const int cp = a > 0 ? s.cls[s.arena[a - 1]] : -1;
@@ -422,35 +559,59 @@ __device__ void arena_pack(const CsrState &s, CsrShared *sh, const CsrGraph &g) 
     __syncthreads();
 }
 
-// Sorted moved vertices, of a panel (shared memory) or of a long row (workspace).
+// Sorted moved vertices: of a panel, in shared memory with the first indices of
+// the new and the old classes as masks, or of a long row, in the workspace (all
+// members of an old class make one new class).
 template <bool LONG>
 struct Moved {
+    const CsrShared *sh;
     const unsigned long long *key;
-    const int *y;
     const int32_t *row;
     int m;
-    // equal for members of one new class, the old class in the high half
-    __device__ __forceinline__ unsigned long long group(int k) const { return LONG ? key[k] >> 32 << 32 : key[k]; }
+    const uint32_t *bits;   // long row: bit k: k is the first of its class (null: not kept)
     __device__ __forceinline__ int cls(int k) const { return (int)(key[k] >> 32); }
-    __device__ __forceinline__ int vertex(int k) const { return LONG ? row[key[k] & 0xFFFFFFFFu] : y[k]; }
-    // the first index after k / the first index at or before k of the run of equal `what`
-    template <typename F>
-    __device__ __forceinline__ int run_end(int k, F what) const {
-        const auto x = what(k);
-        int lo = k, st = 1;   // lo is in the run
-        while (lo + st < m && what(lo + st) == x) lo += st, st *= 2;
-        for (; st > 0; st >>= 1)
-            if (lo + st < m && what(lo + st) == x) lo += st;
-        return lo + 1;
+    __device__ __forceinline__ int vertex(int k) const { return LONG ? row[key[k] & 0xFFFFFFFFu] : sh->y2[k]; }
+    __device__ __forceinline__ bool first(int k) const {   // of its old class
+        return LONG ? k == 0 || cls(k - 1) != cls(k) : (sh->cstart[k >> 5] >> (k & 31)) & 1u;
     }
-    template <typename F>
-    __device__ __forceinline__ int run_start(int k, F what) const {
-        const auto x = what(k);
+    // the first index of k's new class; of its old one; the first index after its new one
+    __device__ __forceinline__ int group_start(int k) const { return LONG ? key_start(k) : bit_at_or_before(sh->gstart, k); }
+    __device__ __forceinline__ int class_start(int k) const { return LONG ? key_start(k) : bit_at_or_before(sh->cstart, k); }
+    __device__ __forceinline__ int group_end(int k) const {
+        if (LONG && !bits) {
+            const int c = cls(k);
+            int lo = k, st = 1;   // lo is in the class
+#pragma unroll 1
+            while (lo + st < m && cls(lo + st) == c) lo += st, st *= 2;
+#pragma unroll 1
+            for (; st > 0; st >>= 1)
+                if (lo + st < m && cls(lo + st) == c) lo += st;
+            return lo + 1;
+        }
+        const uint32_t *starts = LONG ? bits : sh->gstart;
+        int w = k >> 5;
+        uint32_t b = starts[w] & (0xFFFFFFFEu << (k & 31));
+#pragma unroll 1
+        while (!b && 32 * ++w < m) b = starts[w];
+        return b ? 32 * w + __ffs(b) - 1 : m;
+    }
+    __device__ __forceinline__ int key_start(int k) const {
+        if (bits) return bit_at_or_before(bits, k);
+        const int c = cls(k);
         int hi = k, st = 1;
-        while (hi - st >= 0 && what(hi - st) == x) hi -= st, st *= 2;
+#pragma unroll 1
+        while (hi - st >= 0 && cls(hi - st) == c) hi -= st, st *= 2;
+#pragma unroll 1
         for (; st > 0; st >>= 1)
-            if (hi - st >= 0 && what(hi - st) == x) hi -= st;
+            if (hi - st >= 0 && cls(hi - st) == c) hi -= st;
         return hi;
+    }
+    __device__ __forceinline__ int bit_at_or_before(const uint32_t *bits, int k) const {   // (bit 0 is set)
+        int w = k >> 5;
+        uint32_t b = bits[w] & low_bits((k & 31) + 1);
+#pragma unroll 1
+        while (!b && w > 0) b = bits[--w];
+        return 32 * w + 31 - __clz(b);
     }
 };
 
@@ -460,18 +621,21 @@ struct Moved {
 template <bool LONG>
 __device__ __forceinline__ void move_ids(const CsrState &s, CsrShared *sh, const CsrGraph &g, const Moved<LONG> &mv,
                                          int *sub) {
-    auto grp = [&](int k) { return mv.group(k); };
-    auto cl = [&](int k) { return mv.cls(k); };
+#pragma unroll 1
     for (int k = threadIdx.x; k < mv.m; k += kCsrThreads) {
-        if (k > 0 && mv.group(k - 1) == mv.group(k)) continue;
+        if (mv.group_start(k) != k) continue;
         const int c = mv.cls(k);
-        const bool first = k == 0 || mv.cls(k - 1) != c;
+        const bool first = mv.first(k);
         const int4 rc = s.rec[c];
-        const int e = mv.run_end(k, grp);
-        const bool last = e >= mv.m || mv.cls(e) != c;
+        if (rc.z < 0) {   // the class came to the front in this panel
+            sub[k] = -1;
+            continue;
+        }
+        const int e = mv.group_end(k);
+        const bool last = e >= mv.m || mv.first(e);
         int id = -1;
         if (last) {
-            const int mc = e - mv.run_start(k, cl);
+            const int mc = e - mv.class_start(k);
             if (c == g.n) sh->unl_size -= mc;
             else if (mc == rc.z) id = c;
             else s.rec[c].z = rc.z - mc;
@@ -486,17 +650,17 @@ __device__ __forceinline__ void move_ids(const CsrState &s, CsrShared *sh, const
 }
 template <bool LONG>
 __device__ __forceinline__ void move_members(const CsrState &s, CsrShared *sh, const CsrGraph &g,
-                                             const Moved<LONG> &mv, const int *sub) {
-    auto grp = [&](int k) { return mv.group(k); };
-    const unsigned base = sh->atop;
+                                             const Moved<LONG> &mv, const int *sub, unsigned base) {
+#pragma unroll 1
     for (int k = threadIdx.x; k < mv.m; k += kCsrThreads) {
-        const int sf = mv.run_start(k, grp), id = sub[sf], y = mv.vertex(k);
+        const int sf = mv.group_start(k), id = sub[sf], y = mv.vertex(k);
         s.arena[base + k] = y;
+        if (id < 0) continue;
         s.cls[y] = id;
         if (g.parent) g.parent[y] = sh->piv[LONG ? 0 : 32 - __ffs(~(uint32_t)mv.key[k])];
         if (k != sf) continue;
-        const int c = mv.cls(k), e = mv.run_end(k, grp);
-        const bool last = e >= mv.m || mv.cls(e) != c;
+        const int c = mv.cls(k), e = mv.group_end(k);
+        const bool last = e >= mv.m || mv.first(e);
         s.rec[id].x = (int)(base + k);
         s.rec[id].y = (int)(base + e);
         s.rec[id].z = e - k;
@@ -512,7 +676,7 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
                                                                  int32_t *__restrict__ order, int32_t *__restrict__ pos) {
     extern __shared__ __align__(16) unsigned char smem[];
     CsrShared *sh = reinterpret_cast<CsrShared *>(smem);
-    const int n = g.n, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int n = g.n, t = threadIdx.x, lane = t & 31, warp = warp_index();
     const CsrState s = csr_state_carve(ws, n, max_deg);
     // Every row is read once, when its vertex is in a window, so its first read
     // would be a DRAM miss: pull row_ptr and col into L2 (bulk prefetch, no
@@ -520,10 +684,10 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
     prefetch_range_l2<kCsrThreads>(g.row_ptr, (size_t)(n + 1) * sizeof(int64_t));
     prefetch_range_l2<kCsrThreads>(g.col, (size_t)nnz * sizeof(int32_t));
     auto clear_hash = [&]() {
+#pragma unroll 1
         for (int k = t; k < kHashSize; k += kCsrThreads) {
             sh->hkey[k] = -1;
             sh->hmask[k] = 0u;
-            sh->hfront[k] = 0;
         }
     };
     clear_hash();
@@ -546,6 +710,7 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
     int i = 0;     // numbered vertices
     int cur = 0;   // the front at hand
     const int fp = t - (kCsrThreads - kFrontCap);   // the last threads: position in the front
+    const bool front_warp = warp >= (kCsrThreads - kFrontCap) / 32;
     while (i < n) {
         Front *f = &sh->front[cur], *nf = &sh->front[cur ^ 1];
         if (sh->flen == 0) {
@@ -568,25 +733,59 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
         const int entries = long_row ? 0 : (int)__shfl_sync(kFull, einc, w2 - 1);
         __syncthreads();   // everyone has read the front's length
 
-        uint32_t adj = 0u;
-        if (!long_row) {
-            if (warp == 0) {
-                if (pcls < 0 && fl - w2 < kFrontLow && sh->head_next != n)
-                    front_fill(s, sh, g, f, fl, kFrontLow + w2 - fl);
-            } else {
+        // the classes' members in the front: [start, end) of the one at position p
+        auto front_class = [&](int p, int *cs, int *ce, int len) {
+            *cs = 0;
+            *ce = len;
+#pragma unroll 1
+            for (int w = p >> 5; w >= 0; --w) {
+                const uint32_t b = sh->fstart[w] & (w == (p >> 5) ? low_bits((p & 31) + 1) : kFull);
+                if (b) {
+                    *cs = 32 * w + 31 - __clz(b);
+                    break;
+                }
+            }
+#pragma unroll 1
+            for (int w = p >> 5; w < kFrontCap / 32; ++w) {
+                const uint32_t b = sh->fstart[w] & (w == (p >> 5) ? 0xFFFFFFFEu << (p & 31) : kFull);
+                if (b) {
+                    *ce = min(*ce, 32 * w + __ffs(b) - 1);
+                    break;
+                }
+            }
+        };
+        int r = 1;
+        uint32_t pm = 1u;
+        bool ident = true;
+        // a key's bits in pivot order, the first pivot's highest
+        auto pivot_key = [&](uint32_t k) -> uint32_t {
+            if (ident) return __brev(k);
+            uint32_t v = 0u;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) v |= sh->tab[b][(k >> (4 * b)) & 15u];
+            return v;
+        };
+        if (warp == 0) {
+            // ---- the front is filled for the next panel while the workers do this one's keys, order and sort
+            if (!long_row && pcls < 0 && fl - w2 < kFrontLow && sh->head_next != n)
+                front_fill(s, sh, g, f, fl, kFrontLow + w2 - fl);
+        } else {
+            const int wt = t - 32;
+            uint32_t adj = 0u;
+            if (!long_row) {
+                // ---- keys: an entry of the window's rows per thread
                 if (fp >= 0 && fp < fl) {
                     bool fresh;
                     sh->fslot[fp] = hash_slot(sh, f->v[fp], &fresh);
                 }
-                constexpr int U = (kMaxEntries + kCsrThreads - 33) / (kCsrThreads - 32);
-                constexpr int kStep = kCsrThreads - 32;
+                constexpr int U = (kMaxEntries + kCsrWorkers - 1) / kCsrWorkers;
                 int y[U], c[U], own[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int e = t - 32 + u * kStep;
+                    const int e = wt + u * kCsrWorkers;
                     y[u] = -1;
                     own[u] = 0;
-                    if (e - lane < entries) {
+                    if ((warp - 1) * 32 + u * kCsrWorkers < entries) {
                         own[u] = warp_owner(einc, (unsigned)e);
                         const int64_t at = __shfl_sync(kFull, beg, own[u]) +
                                            (e - (int)__shfl_sync(kFull, einc - (unsigned)deg, own[u]));
@@ -597,7 +796,7 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
                 for (int u = 0; u < U; ++u) c[u] = y[u] >= 0 ? s.cls[y[u]] : kNumberedCls;
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    if (t - 32 - lane + u * kStep >= entries) break;
+                    if ((warp - 1) * 32 + u * kCsrWorkers >= entries) break;
                     bool list = false;
                     int h = 0;
                     if (c[u] != kNumberedCls) {
@@ -613,313 +812,343 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
                     if (list && at < kMaxEntries) {
                         sh->key2[at] = (unsigned long long)(unsigned)c[u] << 32 | (unsigned)h;
                         sh->y2[at] = y[u];
+                        prefetch_l1(&s.rec[c[u]]);   // what move_ids reads
+                        prefetch_l1(&s.freel[max(sh->free_top - 1 - at, 0)]);
                     }
                 }
+                named_barrier(1, kCsrWorkers);
+                adj = lane < w2 ? sh->hmask[sh->fslot[lane]] & ~(1u << lane) : 0u;
+            } else if (pcls >= 0) {   // a long row in a large class: the others go back
+                if (fp >= 1 && fp < fl) s.cls[f->v[fp]] = pcls;
+                if (t == 32) sh->pmore = sh->pmore || fl > 1;
+                named_barrier(1, kCsrWorkers);
+                fl = 1;
             }
-            __syncthreads();
-            fl = sh->flen;
-            adj = lane < w2 ? sh->hmask[sh->fslot[lane]] & ~(1u << lane) : 0u;
-        } else if (pcls >= 0) {   // a long row in a large class: the others go back
-            if (fp >= 1 && fp < fl) s.cls[f->v[fp]] = pcls;
-            __syncthreads();
-            if (t == 0) {
-                sh->pmore = sh->pmore || fl > 1;
-                sh->flen = 1;
-            }
-            __syncthreads();
-            fl = 1;
-        }
-        // key of the front's vertex p (long row: searched in the pivot's row)
-        auto front_key = [&](int p) -> uint32_t {
-            if (!long_row) return sh->hmask[sh->fslot[p]];
-            const int32_t *row = g.col + f->beg[0];
-            const int v = f->v[p];
-            int lo = 0, hi = f->deg[0];
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (row[mid] < v) lo = mid + 1; else hi = mid;
-            }
-            return lo < f->deg[0] && row[lo] == v ? 1u : 0u;
-        };
 
-        // ---- the pivots: window vertices 0..r-1 in order, or what warp 0 finds
-        const uint32_t starts = sh->fstart[0] & low_bits(w2);
-        const bool outside = pcls >= 0 && sh->pmore;   // members of the window's class beyond the front
-        const bool straddle = w2 < fl ? w2 == 32 ? !(sh->fstart[1] & 1u) : !((sh->fstart[0] >> w2) & 1u) : outside;
-        uint32_t ub = 0u;
-        if (straddle && !long_row) {
-            if (outside) ub = kFull;
-            else {   // the class's members in the front beyond the window
-                int ce = fl;
-                for (int w = w2 >> 5; w < kFrontCap / 32 && 32 * w < ce; ++w) {
-                    const uint32_t b = sh->fstart[w] & (w == (w2 >> 5) ? kFull << (w2 & 31) : kFull);
-                    if (b) ce = min(ce, 32 * w + __ffs(b) - 1);
+            // ---- the pivots: window vertices 0..r-1 in order, or what warp 1 finds
+            const uint32_t starts = sh->fstart[0] & low_bits(w2);
+            const bool outside = pcls >= 0 && sh->pmore;   // members of the window's class beyond the front
+            const bool straddle = w2 < fl ? w2 == 32 ? !(sh->fstart[1] & 1u) : !((sh->fstart[0] >> w2) & 1u) : outside;
+            uint32_t ub = 0u;
+            if (straddle && !long_row) {
+                if (outside) ub = kFull;
+                else {   // the class's members in the front beyond the window
+                    int cs, ce;
+                    front_class(w2, &cs, &ce, fl);
+#pragma unroll 1
+                    for (int p = w2 + lane; p < ce; p += 32) ub |= sh->hmask[sh->fslot[p]];
+                    ub = __reduce_or_sync(kFull, ub);
                 }
-                for (int p = w2 + lane; p < ce; p += 32) ub |= sh->hmask[sh->fslot[p]];
-                ub = __reduce_or_sync(kFull, ub);
             }
-        }
-        int mypos = -1, la = -1;   // warp 0
-        bool order_fails = false;
-        int r = long_row ? 1 : panel_in_order(lane, w2, starts, straddle, adj, ub, &order_fails);
-        bool ident = true;
-        if (r < w2 && r < kPanelFew) {   // too few (the same in every warp)
-            if (!order_fails && outside) {
-                __syncthreads();
-                uint32_t any = 0u;
-                for (int k = t; k < sh->lcount; k += kCsrThreads)
-                    if ((int)(sh->key2[k] >> 32) == pcls) any |= sh->hmask[(unsigned)sh->key2[k]];
-                if (fp >= w2 && fp < fl) any |= sh->hmask[sh->fslot[fp]];
-                any = __reduce_or_sync(kFull, any);
-                if (lane == 0 && any) atomicOr(&sh->ub, any);
-                __syncthreads();
-                ub = sh->ub;
+            int mypos = -1, la = -1;   // warp 1
+            if (!long_row) {
+                bool order_fails = false;
                 r = panel_in_order(lane, w2, starts, straddle, adj, ub, &order_fails);
+                if (r < w2 && r < kPanelFew) {   // too few (the same in every warp)
+                    if (!order_fails && outside) {
+                        named_barrier(1, kCsrWorkers);
+                        uint32_t any = 0u;
+#pragma unroll 1
+                        for (int k = wt; k < sh->lcount; k += kCsrWorkers)
+                            if ((int)(sh->key2[k] >> 32) == pcls) any |= sh->hmask[(unsigned)sh->key2[k]];
+                        if (fp >= w2 && fp < fl) any |= sh->hmask[sh->fslot[fp]];
+                        any = __reduce_or_sync(kFull, any);
+                        if (lane == 0 && any) atomicOr(&sh->ub, any);
+                        named_barrier(1, kCsrWorkers);
+                        ub = sh->ub;
+                        r = panel_in_order(lane, w2, starts, straddle, adj, ub, &order_fails);
+                    }
+                    ident = !(order_fails && r < kPanelFew);
+                }
             }
-            ident = !(order_fails && r < kPanelFew);
-        }
-        uint32_t pm = low_bits(r);
-        if (warp == 0) {
-            if (ident) {
-                mypos = lane < r ? lane : -1;
-                const uint32_t before = adj & lanes_below(lane);
-                la = before ? 31 - __clz(before) : -1;
-            } else {
-                r = panel_solve(lane, w2, starts, straddle, adj, ub, &mypos, &la);
-            }
-            const uint32_t taken = __ballot_sync(kFull, mypos >= 0);
-            if (mypos >= 0) sh->piv[mypos] = vk;
-            sh->bit[lane] = mypos >= 0 ? 0x80000000u >> mypos : 0u;
-            __syncwarp();
-            if (mypos >= 0) {
-                order[i + mypos] = vk;
-                if (pos) pos[vk] = i + mypos;
-                if (g.parent) g.parent[vk] = la >= 0 ? sh->piv[la] : f->par[lane];
-                s.cls[vk] = kNumberedCls;
-            }
-            if (lane == 0) {
-                sh->r = r;
-                sh->pivmask = taken;
-                if (pcls >= 0) {   // the large class loses the pivots from its head
-                    const int left = __ffs(~taken) - 1;   // -1: none of 32
-                    const unsigned to = left >= 0 && left < fl ? sh->fat[left] : sh->fat[fl - 1] + 1u;
-                    if (pcls == n) {
-                        sh->unl_size -= r;
-                        sh->unl_cur = (int)to;
-                    } else {
-                        const int sz = s.rec[pcls].z - r;
-                        s.rec[pcls].z = sz;
-                        s.rec[pcls].x = (int)to;
-                        if (sz == 0) {
-                            const int nx = get_next(s, sh, g, pcls);
-                            sh->head_next = nx;
-                            s.rec[nx].w = kHead;
-                            s.freel[sh->free_top++] = pcls;
+            pm = low_bits(r);
+            if (warp == 1) {
+                if (ident) {
+                    mypos = lane < r ? lane : -1;
+                    const uint32_t before = adj & lanes_below(lane);
+                    la = before ? 31 - __clz(before) : -1;
+                } else {
+                    r = panel_solve(lane, w2, starts, straddle, adj, ub, &mypos, &la);
+                }
+                const uint32_t taken = __ballot_sync(kFull, mypos >= 0);
+                if (mypos >= 0) sh->piv[mypos] = vk;
+                sh->bit[lane] = mypos >= 0 ? 0x80000000u >> mypos : 0u;
+                __syncwarp();
+                if (mypos >= 0) {
+                    order[i + mypos] = vk;
+                    if (pos) pos[vk] = i + mypos;
+                    if (g.parent) g.parent[vk] = la >= 0 ? sh->piv[la] : f->par[lane];
+                    s.cls[vk] = kNumberedCls;
+                }
+                if (lane == 0) {
+                    sh->r = r;
+                    sh->pivmask = taken;
+                    if (pcls >= 0) {   // the large class loses the pivots from its head
+                        const int left = __ffs(~taken) - 1;   // -1: none of 32
+                        const unsigned to = left >= 0 && left < fl ? sh->fat[left] : sh->fat[fl - 1] + 1u;
+                        if (pcls == n) {
+                            sh->unl_size -= r;
+                            sh->unl_cur = (int)to;
+                        } else {
+                            const int sz = s.rec[pcls].z - r;
+                            s.rec[pcls].z = sz;
+                            s.rec[pcls].x = (int)to;
+                            if (sz == 0) {
+                                const int nx = get_next(s, sh, g, pcls);
+                                sh->head_next = nx;
+                                s.rec[nx].w = kHead;
+                                s.freel[sh->free_top++] = pcls;
+                            }
                         }
                     }
                 }
             }
-        }
-        if (!ident) {
-            __syncthreads();
-            r = sh->r;
-            pm = sh->pivmask;
-            if (t < 128) {
-                uint32_t v = 0u;
+            if (!ident) {
+                named_barrier(1, kCsrWorkers);
+                pm = sh->pivmask;
+                if (wt < 128) {
+                    uint32_t v = 0u;
 #pragma unroll
-                for (int b = 0; b < 4; ++b)
-                    if ((t >> b) & 1) v |= sh->bit[((t >> 4) << 2) + b];
-                sh->tab[t >> 4][t & 15] = v;
-            }
-            __syncthreads();
-        }
-        // a key's bits in pivot order, the first pivot's highest
-        auto pivot_key = [&](uint32_t k) -> uint32_t {
-            if (ident) return __brev(k);
-            uint32_t v = 0u;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) v |= sh->tab[b][(k >> (4 * b)) & 15u];
-            return v;
-        };
-
-        // ---- the moved vertices of the listed classes; the front's labels
-        auto append = [&](bool keep, int c, uint32_t pk, int y) {
-            const unsigned lm = __ballot_sync(kFull, keep);
-            int at = 0;
-            if (lane == 0 && lm) at = atomicAdd(&sh->m, __popc(lm));
-            at = __shfl_sync(kFull, at, 0) + __popc(lm & lanes_below(lane));
-            if (keep && at < kMaxEntries) {
-                sh->key[at] = (unsigned long long)(unsigned)c << 32 | (unsigned)~pk;
-                sh->y[at] = y;
-            }
-        };
-        if (!long_row) {
-            const int lc = sh->lcount;
-            for (int k0 = warp * 32; k0 < lc; k0 += kCsrThreads) {
-                const int k = k0 + lane;
-                unsigned long long e = 0ull;
-                uint32_t mk = 0u;
-                if (k < lc) {
-                    e = sh->key2[k];
-                    if (!sh->hfront[(unsigned)e]) mk = sh->hmask[(unsigned)e] & pm;
+                    for (int b = 0; b < 4; ++b)
+                        if ((wt >> b) & 1) v |= sh->bit[((wt >> 4) << 2) + b];
+                    sh->tab[wt >> 4][wt & 15] = v;
                 }
-                append(mk != 0u, (int)(e >> 32), pivot_key(mk), k < lc ? sh->y2[k] : 0);
+                named_barrier(1, kCsrWorkers);
             }
-        }
-        if (fp >= lane) {   // the front's warps
-            const bool left = fp < fl && !(fp < 32 && ((pm >> fp) & 1u));
-            uint32_t k = left ? front_key(fp) & pm : 0u;
-            if (pcls >= 0) {   // the rest of a large class goes back (a long row left none)
+
+            // ---- the moved vertices of the listed classes; the front's labels
+            auto append = [&](bool keep, int c, uint32_t pk, int y) {
+                const unsigned lm = __ballot_sync(kFull, keep);
+                int at = 0;
+                if (lane == 0 && lm) at = atomicAdd(&sh->m, __popc(lm));
+                at = __shfl_sync(kFull, at, 0) + __popc(lm & lanes_below(lane));
+                if (keep && at < kMaxEntries) {
+                    sh->key[at] = (unsigned long long)(unsigned)c << 32 | (unsigned)~pk;
+                    sh->y[at] = y;
+                }
+            };
+            if (!long_row) {
+                const int lc = sh->lcount;
+#pragma unroll 1
+                for (int k0 = (warp - 1) * 32; k0 < lc; k0 += kCsrWorkers) {
+                    const int k = k0 + lane;
+                    unsigned long long e = 0ull;
+                    uint32_t mk = 0u;
+                    if (k < lc) {
+                        e = sh->key2[k];
+                        mk = sh->hmask[(unsigned)e] & pm;
+                        if (mk && s.rec[(int)(e >> 32)].z == 1) {   // a class of one: it keeps its place
+                            if (g.parent) g.parent[sh->y2[k]] = ident ? f->v[31 - __clz(mk)] : sh->piv[32 - __ffs(pivot_key(mk))];
+                            mk = 0u;
+                        }
+                    }
+                    append(mk != 0u, (int)(e >> 32), pivot_key(mk), k < lc ? sh->y2[k] : 0);
+                }
+            }
+            if (front_warp && pcls >= 0) {   // the front's warps: the rest of a large class goes back (a long row left none)
+                const bool left = fp < fl && !(fp < 32 && ((pm >> fp) & 1u));
+                const uint32_t k = left ? sh->hmask[sh->fslot[fp]] & pm : 0u;
                 if (left && k == 0u) s.cls[f->v[fp]] = pcls;
                 append(k != 0u, pcls, pivot_key(k), left ? f->v[fp] : 0);
-            } else if (left) {
-                const uint32_t pk = pivot_key(k);
-                sh->fck[fp] = ~pk;
-                if (k) f->par[fp] = ident ? f->v[31 - __clz(k)] : sh->piv[32 - __ffs(pk)];
             }
-        }
-        if (long_row) {
-            const int64_t rb = f->beg[0];
-            const int d = f->deg[0];
-            const int64_t p2 = pow2_at_least(d);
-            __syncthreads();   // the pivot's cls
-            for (int64_t k = t; k < p2; k += kCsrThreads) {
-                unsigned long long e = ~0ull;
-                if (k < d) {
-                    const int c = s.cls[g.col[rb + k]];
-                    if (c >= 0) e = (unsigned long long)(unsigned)c << 32 | (unsigned long long)k;
-                }
-                s.skey[k] = e;
-                const unsigned lm = __ballot_sync(kFull, e != ~0ull);   // p2 is a multiple of the CTA
-                if (lm && lane == 0) atomicAdd(&sh->m, __popc(lm));
+            if (!long_row) {
+                named_barrier(1, kCsrWorkers);
+                panel_sort_moved(sh, sh->m);   // by (class, label, id)
             }
         }
         __syncthreads();
-        const int m = sh->m;
-
-        // ---- sorted by (class, label, id)
-        const unsigned long long *skey = sh->key2;
-        const int *sy = sh->y2;
-        if (long_row) {
-            cta_sort_keys_tiled(s.skey, pow2_at_least(f->deg[0]), sh->key, kMaxEntries);   // deg > kMaxEntries
-        } else if (m <= 512) {   // ranks by counting, as many lanes per vertex as there are
-            const int lg = m <= 32 ? 5 : m <= 64 ? 4 : m <= 128 ? 3 : m <= 256 ? 2 : 1;
-            const int e = t >> lg, step = 1 << lg;
-            if ((warp * 32) >> lg < m) {
-                const unsigned long long ke = e < m ? sh->key[e] : 0ull;
-                const int ye = e < m ? sh->y[e] : 0;
-                int rank = 0;
-#pragma unroll 4
-                for (int k = t & (step - 1); k < m; k += step) {
-                    const unsigned long long kk = sh->key[k];
-                    rank += kk < ke || (kk == ke && sh->y[k] < ye) ? 1 : 0;
-                }
-                for (int o = 1; o < step; o <<= 1) rank += __shfl_xor_sync(kFull, rank, o);
-                if (e < m && (t & (step - 1)) == 0) {
-                    sh->key2[rank] = ke;
-                    sh->y2[rank] = ye;
-                }
-            }
-        } else {
-            int p2 = 1024;
-            if (m > 1024) p2 = 2048;
-            for (int e = m + t; e < p2; e += kCsrThreads) {
-                sh->key[e] = ~0ull;
-                sh->y[e] = 0;
-            }
-            __syncthreads();
-            for (int k = 2; k <= p2; k <<= 1)
-                for (int j = k >> 1; j > 0; j >>= 1) {
-                    const int e = t;
-                    if (e < p2 / 2) {
-                        const int lo = ((e & ~(j - 1)) << 1) | (e & (j - 1)), hi = lo | j;
-                        const unsigned long long a = sh->key[lo], b = sh->key[hi];
-                        const int ya = sh->y[lo], yb = sh->y[hi];
-                        if ((a > b || (a == b && ya > yb)) == ((lo & k) == 0)) {
-                            sh->key[lo] = b;
-                            sh->key[hi] = a;
-                            sh->y[lo] = yb;
-                            sh->y[hi] = ya;
-                        }
-                    }
-                    __syncthreads();
-                }
-            skey = sh->key;
-            sy = sh->y;
-        }
-        // ---- the front after the panel: each class's members by label
+        r = sh->r;
+        pm = sh->pivmask;
+        if (warp == 0) ident = false;   // (no labels needed)
+        int m = sh->m, unl = 0;
+        if (pcls < 0) fl = sh->flen;
         const int fl2 = pcls >= 0 ? 0 : fl - r;
-        if (pcls < 0 && fp >= 0 && fp < fl && !(fp < 32 && ((pm >> fp) & 1u))) {
-            int cs = 0, ce = fl;
-            for (int w = fp >> 5; w >= 0; --w) {
-                const uint32_t b = sh->fstart[w] & (w == (fp >> 5) ? low_bits((fp & 31) + 1) : kFull);
-                if (b) {
-                    cs = 32 * w + 31 - __clz(b);
-                    break;
-                }
-            }
-            for (int w = fp >> 5; w < kFrontCap / 32; ++w) {
-                const uint32_t b = sh->fstart[w] & (w == (fp >> 5) ? 0xFFFFFFFEu << (fp & 31) : kFull);
-                if (b) {
-                    ce = min(ce, 32 * w + __ffs(b) - 1);
-                    break;
-                }
-            }
-            int np = cs - __popc(pm & low_bits(cs));
-            const uint32_t ck = sh->fck[fp];
-            for (int q = cs; q < ce; ++q) {
-                if (q < 32 && ((pm >> q) & 1u)) continue;
-                const uint32_t cq = sh->fck[q];
-                np += cq < ck || (cq == ck && q < fp) ? 1 : 0;
-            }
-            nf->v[np] = f->v[fp];
-            nf->par[np] = f->par[fp];
-            nf->beg[np] = f->beg[fp];
-            nf->deg[np] = f->deg[fp];
-            sh->nck[np] = ck;
-            sh->ncs[np] = cs;
-        }
-        __syncthreads();
 
-        // ---- new classes
-        if (fp >= lane) {
+        // ---- the front after the panel: each class's members by label (the last warps)
+        if (front_warp) {
+            const bool left = pcls < 0 && fp < fl && !(fp < 32 && ((pm >> fp) & 1u));
+            uint32_t ck = 0u;
+            if (left) {
+                const int v = f->v[fp];
+                uint32_t k;
+                if (long_row) {   // searched in the pivot's row
+                    const int32_t *row = g.col + f->beg[0];
+                    int lo = 0, hi = f->deg[0];
+#pragma unroll 1
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if (row[mid] < v) lo = mid + 1; else hi = mid;
+                    }
+                    k = lo < f->deg[0] && row[lo] == v ? 1u : 0u;
+                } else {
+                    k = hash_key(sh, v) & pm;
+                }
+                const uint32_t pk = pivot_key(k);
+                ck = ~pk;
+                sh->fck[fp] = ck;
+                if (k) f->par[fp] = sh->piv[32 - __ffs(pk)];
+            }
+            named_barrier(2, kFrontCap);
+            if (left) {
+                int cs, ce;
+                front_class(fp, &cs, &ce, fl);
+                int np = cs - __popc(pm & low_bits(cs));
+#pragma unroll 1
+                for (int q = cs; q < ce; ++q) {
+                    if (q < 32 && ((pm >> q) & 1u)) continue;
+                    const uint32_t cq = sh->fck[q];
+                    np += cq < ck || (cq == ck && q < fp) ? 1 : 0;
+                }
+                nf->v[np] = f->v[fp];
+                nf->par[np] = f->par[fp];
+                nf->beg[np] = f->beg[fp];
+                nf->deg[np] = f->deg[fp];
+                sh->nck[np] = ck;
+                sh->ncs[np] = cs;
+            }
+            named_barrier(2, kFrontCap);
             const bool st = fp < fl2 &&
                             (fp == 0 || sh->ncs[fp] != sh->ncs[fp - 1] || sh->nck[fp] != sh->nck[fp - 1]);
             const uint32_t b = __ballot_sync(kFull, st);
             if (lane == 0) sh->fstart[fp >> 5] = b;
         }
+
+        // a class of one vertex: moving it changes nothing but its last adjacent pivot
+        auto single = [&](int c) -> bool { return s.rec[c].z == 1; };
+        // ---- a long row: the vertices without a numbered neighbour come in id order already, the others are sorted
+        // by (class, row position), in shared memory when they fit
+        const unsigned long long *lkey = nullptr;
+        if (long_row) {
+            const int64_t rb = f->beg[0];
+            const int d = f->deg[0];
+            int *kept = s.subid;   // the class of the row's k-th vertex when it is to be sorted
+#pragma unroll 1
+            for (int k0 = 32 * warp; k0 < d; k0 += kCsrThreads) {
+                const int k = k0 + lane;
+                const int y = k < d ? g.col[rb + k] : 0;
+                int c = k < d ? s.cls[y] : kNumberedCls;
+                if (c >= 0 && c != n && single(c)) {
+                    if (g.parent) g.parent[y] = f->v[0];
+                    c = kNumberedCls;
+                }
+                const unsigned um = __ballot_sync(kFull, c == n), lm = __ballot_sync(kFull, c >= 0 && c != n);
+                if (lane == 0 && um) atomicAdd(&sh->lcount, __popc(um));
+                if (lane == 0 && lm) atomicAdd(&sh->m, __popc(lm));
+                if (k < d) kept[k] = c != n ? c : kNumberedCls;
+            }
+            __syncthreads();
+            m = sh->m;
+            unl = sh->lcount;
+            // the new members' place at the arena's end, and a buffer after it
+            if ((int64_t)s.cap - sh->atop < 3 * ((int64_t)m + unl) + 2) {   // the same for all threads
+                __syncthreads();
+                arena_pack(s, sh, g);
+            }
+            int *const after = (int *)s.arena + sh->atop + (unsigned)(m + unl);
+            lkey = sort_long_row(sh, kept, d, m, n,
+                                 reinterpret_cast<unsigned long long *>((reinterpret_cast<uintptr_t>(after) + 7) & ~uintptr_t(7)),
+                                 (unsigned long long *)s.skey);
+        }
+
+        // ---- new classes
         // nothing in the list but vertices that had no numbered neighbour: what the panel met goes to the front
-        const bool to_front = !long_row && m > 0 && fl2 + m <= kFrontCap && sh->head_next == n;
-        const Moved<false> mv{skey, sy, nullptr, m};
-        const Moved<true> ml{s.skey, nullptr, g.col + f->beg[0], m};
+        const bool to_front = !long_row && m > 0 && fl2 + m <= kFrontCap && sh->head_next == n &&
+                              (int)(sh->key2[0] >> 32) == n;
+        const Moved<false> mv{sh, sh->key2, nullptr, m, nullptr};
+        uint32_t *lbits = reinterpret_cast<uint32_t *>(sh->y);   // y, y2 and sub
+        const bool keep_bits = long_row && m <= 3 * 32 * kMaxEntries;
+        const Moved<true> ml{sh, lkey, g.col + f->beg[0], m, keep_bits ? lbits : nullptr};
+        if (keep_bits)
+#pragma unroll 1
+            for (int k0 = 32 * warp; k0 < m; k0 += kCsrThreads) {
+                const int k = k0 + lane;
+                const uint32_t cb =
+                    __ballot_sync(kFull, k < m && (k == 0 || lkey[max(k - 1, 0)] >> 32 != lkey[k] >> 32));
+                if (lane == 0) lbits[k0 >> 5] = cb;
+            }
+        if (!long_row && !to_front)
+#pragma unroll 1
+            for (int k0 = 32 * warp; k0 < m; k0 += kCsrThreads) {
+                const int k = k0 + lane;
+                const unsigned long long x = k < m ? sh->key2[k] : 0ull, px = k > 0 && k < m ? sh->key2[k - 1] : 0ull;
+                const uint32_t gb = __ballot_sync(kFull, k < m && (k == 0 || x != px));
+                const uint32_t cb = __ballot_sync(kFull, k < m && (k == 0 || x >> 32 != px >> 32));
+                if (lane == 0) {
+                    sh->gstart[k0 >> 5] = gb;
+                    sh->cstart[k0 >> 5] = cb;
+                }
+            }
+        __syncthreads();
         if (!to_front) {
             if (long_row) move_ids(s, sh, g, ml, (int *)s.subid);
             else move_ids(s, sh, g, mv, sh->sub);
         }
+        if (t == 0 && unl > 0) {   // the new class before the last one
+            const int id = s.freel[atomicSub(&sh->free_top, 1) - 1], before = s.rec[n].w;
+            s.rec[id].w = before;
+            set_next(s, sh, g, before, id);
+            set_next(s, sh, g, id, n);
+            s.rec[n].w = id;
+            sh->unl_size -= unl;
+            sh->unl_id = id;
+        }
+        unsigned atop = sh->atop;
         clear_hash();
         __syncthreads();
-        if (to_front) {
-            if (t < m) {
-                const int p = fl2 + t, y = sy[t];
-                front_put(sh, nf, g, p, y, sh->piv[32 - __ffs(~(uint32_t)skey[t])]);
-                s.cls[y] = kFrontCls;
-                if (t == 0 || skey[t] != skey[t - 1]) atomicOr(&sh->fstart[p >> 5], 1u << (p & 31));
-            }
-        } else if (m > 0) {
-            if (s.cap - sh->atop < (unsigned)m) arena_pack(s, sh, g);   // the same for all threads
-            if (long_row) move_members(s, sh, g, ml, (int *)s.subid);
-            else move_members(s, sh, g, mv, sh->sub);
-        }
-        __syncthreads();
-        if (t == 0) {
+        if (t == 0) {   // (what the threads still need of these they hold)
             sh->flen = fl2 + (to_front ? m : 0);
             sh->pcls = -1;
             sh->pmore = 0;
-            if (to_front) sh->unl_size -= m;
-            else sh->atop += (unsigned)m;
             sh->lcount = 0;
             sh->m = 0;
             sh->ub = 0u;
+            if (to_front) sh->unl_size -= m;
+        }
+        if (to_front) {
+            if (t < m) {
+                const int p = fl2 + t, y = sh->y2[t];
+                const unsigned long long k = sh->key2[t];
+                front_put(nf, p, y, sh->piv[32 - __ffs(~(uint32_t)k)], g.row_ptr[y], g.row_ptr[y + 1]);
+                s.cls[y] = kFrontCls;
+                if (t == 0 || k != sh->key2[t - 1]) atomicOr(&sh->fstart[p >> 5], 1u << (p & 31));
+            }
+        } else if (m + unl > 0) {
+            if (s.cap - atop < (unsigned)(m + unl)) {   // the same for all threads (a long row has its room)
+                arena_pack(s, sh, g);
+                atop = sh->atop;
+                __syncthreads();
+            }
+            if (t == 0) sh->atop = atop + (unsigned)(m + unl);
+            if (long_row) move_members(s, sh, g, ml, (int *)s.subid, atop);
+            else move_members(s, sh, g, mv, sh->sub, atop);
+            if (unl > 0) {   // those without a numbered neighbour, in row order
+                const int64_t rb = f->beg[0];
+                const int d = f->deg[0], id = sh->unl_id, x = f->v[0];
+                const unsigned out = atop + (unsigned)m;
+                unsigned done = 0u;
+#pragma unroll 1
+                for (int k0 = 0; k0 < d; k0 += kCsrThreads) {
+                    const int k = k0 + t, y = k < d ? g.col[rb + k] : -1;
+                    const bool in = k < d && s.cls[y] == n;
+                    const unsigned lm = __ballot_sync(kFull, in);
+                    if (lane == 0) sh->scan[warp] = __popc(lm);
+                    __syncthreads();
+                    const int wc = lane < kCsrThreads / 32 ? sh->scan[lane] : 0;
+                    const int ahead = __reduce_add_sync(kFull, lane < warp ? wc : 0);
+                    if (in) {
+                        s.arena[out + done + ahead + __popc(lm & lanes_below(lane))] = y;
+                        s.cls[y] = id;
+                        if (g.parent) g.parent[y] = x;
+                    }
+                    done += __reduce_add_sync(kFull, wc);
+                    __syncthreads();
+                }
+                if (t == 0) {
+                    s.rec[id].x = (int)out;
+                    s.rec[id].y = (int)(out + unl);
+                    s.rec[id].z = unl;
+                }
+            }
         }
         i += r;
         cur ^= 1;
