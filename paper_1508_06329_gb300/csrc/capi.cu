@@ -770,6 +770,7 @@ int run_mcs_dense(cg_context *ctx, const cg_dense *g, int32_t *order_out, int32_
     const size_t o_parent = cv.take<int32_t>(n);
     const size_t o_key = cv.take<unsigned long long>(2);
     const size_t o_emask = cv.take<uint32_t>(res ? earlier_mask_words(n) : 0);
+    const size_t o_left = cv.take<unsigned char>(mcs_workspace_bytes(n));
     int rc;
     if ((rc = ensure_ws(ctx, cv.off))) return rc;
     int32_t *order = order_out ? order_out : at<int32_t>(ctx, o_order);
@@ -778,8 +779,8 @@ int run_mcs_dense(cg_context *ctx, const cg_dense *g, int32_t *order_out, int32_
     const DenseDesc d = desc_of(g, 0, 0);
     if (n > 0) {
         PhaseTimer pt(ctx, &ctx->ev_lex, stream);
-        if ((rc = mcs_dense_launch(d, order, pos, stream))) return rc;
-        ctx->launches += 1;
+        if ((rc = mcs_dense_launch(d, order, pos, at<void>(ctx, o_left), stream))) return rc;
+        ctx->launches += mcs_workspace_bytes(n) ? 2 : 1;
     }
     if (!res) return CG_OK;
     PhaseTimer pt(ctx, &ctx->ev_check, stream);

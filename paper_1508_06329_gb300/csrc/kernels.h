@@ -27,7 +27,7 @@ int lexbfs_dense_plan(int n_max, int threads_override, LexPlan *plan);
 // work_counter: device int, zeroed by the launcher (dynamic graph hand-out).
 // ppos (nullable, packed by vbase) receives the parents by position:
 // ppos[i] = p(order[i]), -1 when it has no earlier neighbour.  keys (nullable)
-// is set, on the stream after the search, to the check's initial keys:
+// is set by the search to the check's initial keys:
 // keys[0..count) = "no violation", keys[count] = keys[count + 1] = 0.
 // emask (nullable): the search also writes each graph's earlier-than masks
 // E_b (b >= 1; row b at emask + ebase + b * mask_stride(n): the vertices
@@ -129,7 +129,8 @@ int sweep_order_launch(const DenseDesc &d, const LexPlan &plan, void *gstate, in
                        int32_t *order, int32_t *pos, int num_sms, cudaStream_t stream);
 
 // ---- dense MCS (mcs_dense.cu): one CTA, n <= 65520
-int mcs_dense_launch(DenseDesc d, int32_t *order, int32_t *pos, cudaStream_t stream);
+size_t mcs_workspace_bytes(int n);   // 16-byte aligned
+int mcs_dense_launch(DenseDesc d, int32_t *order, int32_t *pos, void *ws, cudaStream_t stream);
 
 // ---- CSR LexBFS (lexbfs_csr.cu): one CTA per graph (warp 0 walks the steps), state in `ws`
 size_t lexbfs_csr_workspace_bytes(int64_t n, int64_t max_deg);
