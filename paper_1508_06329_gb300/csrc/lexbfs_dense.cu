@@ -23,7 +23,8 @@ __global__ void __launch_bounds__(T) lexbfs_dense_kernel(const DenseDesc *__rest
                                                          int count, int32_t *__restrict__ order,
                                                          int32_t *__restrict__ pos, int32_t *ppos,
                                                          unsigned char *gstate, size_t gstate_stride,
-                                                         int *work_counter, uint32_t *emask, int cap) {
+                                                         int *work_counter, uint32_t *emask, int cap,
+                                                         unsigned long long *keys) {
     extern __shared__ __align__(16) unsigned char smem[];
     PanelScalars *sc = reinterpret_cast<PanelScalars *>(smem);
 #ifdef CG_BOUNDS_CHECK
@@ -32,6 +33,8 @@ __global__ void __launch_bounds__(T) lexbfs_dense_kernel(const DenseDesc *__rest
         cg_dbg_inject_code = 0u;
     }
 #endif
+    if (keys && blockIdx.x == 0)   // the check's initial keys: "no violation", then its CTA counter and error word
+        for (int k = threadIdx.x; k < count + 2; k += T) keys[k] = k < count ? ~0ull : 0ull;
     for (;;) {
         if (threadIdx.x == 0) sc->next_graph = count == 1 ? (int)blockIdx.x : atomicAdd(work_counter, 1);
         __syncthreads();
@@ -60,11 +63,7 @@ int launch_variant(const LexPlan &plan, const DenseDesc *descs, DenseDesc single
     if (count > 1) CG_CUDA_TRY(cudaMemsetAsync(work_counter, 0, sizeof(int), stream));
     kern<<<ctas, T, plan.smem_bytes, stream>>>(descs, single, count, order, pos, ppos,
                                                static_cast<unsigned char *>(gstate), plan.gstate_bytes, work_counter,
-                                               emask, plan.sort_cap);
-    if (keys) {   // the check's initial keys: "no violation", then the CTA counter and error word
-        CG_CUDA_TRY(cudaMemsetAsync(keys, 0xFF, sizeof(unsigned long long) * count, stream));
-        CG_CUDA_TRY(cudaMemsetAsync(keys + count, 0, 2 * sizeof(unsigned long long), stream));
-    }
+                                               emask, plan.sort_cap, keys);
     CG_LAUNCH_CHECK("lexbfs_dense_kernel");
     CG_DEBUG_CHECK(stream, "lexbfs_dense_kernel");
     return CG_OK;
@@ -89,9 +88,9 @@ int lexbfs_dense_plan(int n_max, int threads_override, LexPlan *plan) {
     p.sort_cap = panel_sort_cap(n, room(p.state));
     p.smem_bytes = kPanelScalarBytes + panel_state_bytes(n, p.state) + panel_sort_bytes(p.sort_cap);
     p.gstate_bytes = panel_global_bytes(n, p.state);
-    // measured on GB300 (us): n = 1,000 208 with 256 threads, 253 with 128; n = 16,384 pair 4,350 with
-    // 512, 4,570 with 1,024, 5,790 with 256
-    int th = n <= 4096 ? 256 : 512;
+    // measured on GB300 (us) with 128 / 256 / 512 threads: n = 1,000 226 / 187 / 210, 2,048 512 / 393 / 390,
+    // 4,096 1,147 / 813 / 686; the pair of n = 16,384 with 512 4,350, with 1,024 4,570
+    int th = n <= 2048 ? 256 : 512;
     if (threads_override) th = threads_override;
     if (p.state != kStateSmem) th = 1024;
     if (th != 128 && th != 256 && th != 512 && th != 1024)

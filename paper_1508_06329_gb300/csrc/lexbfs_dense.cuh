@@ -104,6 +104,7 @@ constexpr int kSortCapMax = 4096;
 // the state leaves less room (bytes: shared memory available for them).
 __host__ __device__ inline int panel_sort_cap(int n, size_t bytes) {
     int cap = kSortCapMax;
+#pragma unroll 1
     while (cap > 64 && (cap / 2 >= n || (size_t)cap * 12 > bytes)) cap /= 2;
     return cap;
 }
@@ -254,6 +255,12 @@ __device__ __forceinline__ void panel_load_rows(const uint32_t *__restrict__ col
     }
 }
 
+// The thread's warp, from a shuffle: the compiler then knows that it is the same
+// in all lanes, and that loops and branches on it keep the warp together.  Without
+// that every shuffle and vote in them carries a branch and code for a warp that has
+// come apart.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ uint32_t lanes_below(int lane) { return (1u << lane) - 1u; }
 __device__ __forceinline__ uint32_t low_bits(int k) { return k >= 32 ? 0xFFFFFFFFu : (1u << k) - 1u; }
 
@@ -276,6 +283,7 @@ __device__ __forceinline__ int panel_in_order(int lane, int w2, uint32_t starts,
     const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, adj, 1);
     const uint32_t f1 = __ballot_sync(0xFFFFFFFFu, straddle && lane < w2 && !above && loses(ub));
     uint32_t f0 = 0u;
+#pragma unroll 1
     for (uint32_t larger = __ballot_sync(0xFFFFFFFFu, lane + 1 < w2 && !((starts >> lane) & 2u) && loses(next)); larger;
          larger &= larger - 1u) {
         const int y = __ffs(larger);   // the lane after the one that loses to it
@@ -301,6 +309,7 @@ __device__ __forceinline__ int panel_solve(int lane, int w2, uint32_t starts, bo
     const uint32_t cs = straddle ? undone & (0xFFFFFFFFu << (31 - __clz(starts))) : 0u;
     uint32_t key = 0u, front = 0u, fkey = 0u, ubkey = 0u, cls = 0u;
     int r = 0, mypos = -1, la = -1;
+#pragma unroll 1
     while (undone) {
         if (!front) {   // the top class's members with the largest label
             if (!(cls & undone)) {
@@ -343,7 +352,7 @@ template <int T, bool MINMAX>
 __device__ __forceinline__ int panel_scan(PanelScalars *sc, int &a, int &b, int &c) {
     constexpr int NW = T / 32;
     constexpr int kBig = 0x7FFFFFFF;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = warp_index();
     int ia = a, ib = b, ic = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -383,8 +392,11 @@ __device__ __forceinline__ int panel_scan(PanelScalars *sc, int &a, int &b, int 
 // to 32 stay inside a warp's 64 elements and need no CTA barrier.
 template <int T>
 __device__ __forceinline__ void panel_sort(unsigned long long *a, int p) {
+#pragma unroll 1
     for (int k = 2; k <= p; k <<= 1)
+#pragma unroll 1
         for (int j = k >> 1; j > 0; j >>= 1) {
+#pragma unroll 1
             for (int e = threadIdx.x; e < p / 2; e += T) {
                 const int lo = ((e & ~(j - 1)) << 1) | (e & (j - 1)), hi = lo | j;
                 const unsigned long long x = a[lo], y = a[hi];
@@ -405,6 +417,7 @@ template <int T, typename Arr>
 __device__ __forceinline__ void panel_write_mask(uint32_t *emask, int b, int n, const Arr &numbered) {
     const int wn = (n + 31) >> 5, es = mask_stride(n);
     uint32_t *e = emask + (size_t)b * es;
+#pragma unroll 1
     for (int w = threadIdx.x; w < es; w += T) e[w] = w < wn ? numbered[w] : 0u;
 }
 
@@ -425,10 +438,12 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
     // once per panel is bound by instruction fetch, and the same passes unrolled
     // eight times took 4,096 small graphs from 1.5 to 2.5 ms.
     constexpr int G = T >= 512 ? 8 : 1;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, lane = t & 31, warp = warp_index();
     const int wn = (n + 31) >> 5;
 
+#pragma unroll 1
     for (int q = t; q < 32 * wn; q += T) st.perm[q] = (Id)q;   // positions past n too: they are read in eights
+#pragma unroll 1
     for (int w = t; w < wn; w += T) {
         st.start[w] = w == 0 ? 1u : 0u;
         st.diff[w] = 0u;
@@ -454,6 +469,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
         reinterpret_cast<uint32_t *>(sc->row4)[lane] = 4u * (uint32_t)vk;
         __syncwarp();
         // ---- keys: a word of vertices per thread and pass
+#pragma unroll 1
         for (int wb = warp * 32; wb < wn; wb += T) {
             const int w = wb + lane;
             const bool on = w < wn && st.numbered[w] != kAll;   // some vertex still to come
@@ -523,6 +539,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 }
                 __syncthreads();
                 const int q0 = i + w2;
+#pragma unroll 1
                 for (int w = (q0 >> 5) + t; w < wn; w += T) {
                     const uint32_t b = st.start[w] & (w == (q0 >> 5) ? kAll << (q0 & 31) : kAll);
                     if (b) {
@@ -533,6 +550,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 __syncthreads();
                 const int ce = sc->cend;
                 uint32_t any = 0u;
+#pragma unroll 1
                 for (int q = q0 + t; q < ce; q += T) any |= st.key[key_slot(st.perm[q])];
                 any = __reduce_or_sync(kAll, any);
                 if (lane == 0 && any) atomicOr(&sc->ub, any);
@@ -567,6 +585,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
         for (;;) {
             i2 = i + r;
             if (!ident)
+#pragma unroll 1
                 for (int e = t; e < 128; e += T) {
                     uint32_t v = 0u;
 #pragma unroll
@@ -575,6 +594,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                     sc->tab[e >> 4][e & 15] = v;
                 }
             bool differ = false;
+#pragma unroll 1
             for (int c = warp ? (i2 & ~255) + (warp - 1) * 256 : n; c < n; c += (T - 32) * 8) {   // (warp 0: commit)
                 const int q0 = c + 8 * lane;
                 uint32_t k[8], kp = 0u;
@@ -615,6 +635,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
             // ---- positions of the classes that split (thread t: words [wa, wb) of positions)
             const int kw = (wn + T - 1) / T, wa = min(t * kw, wn), wb = min(wa + kw, wn);
             int ds = 0, lm = -1, nm = 0x7FFFFFFF;
+#pragma unroll 1
             for (int w = wa; w < wb; ++w) {
                 const uint32_t b = st.start[w];
                 if (w >= pw) ds += __popc(st.diff[w]);
@@ -624,6 +645,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 }
             }
             const int dtotal = panel_scan<T, true>(sc, ds, lm, nm);
+#pragma unroll 1
             for (int w = wa; w < wb; ++w) {
                 const uint32_t b = st.start[w];
                 st.dpre[w] = ds;
@@ -632,6 +654,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 st.last[w] = lm;
             }
             nm = min(nm, n);
+#pragma unroll 1
             for (int w = wb - 1; w >= wa; --w) {
                 const uint32_t b = st.start[w];
                 if (b) nm = 32 * w + __ffs(b) - 1;
@@ -645,6 +668,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 return w < pw ? 0 : st.dpre[w] + __popc(st.diff[w] & lanes_below(q & 31));
             };
             int nzs = 0;
+#pragma unroll 1
             for (int w = wa; w < wb; ++w) {
                 uint32_t f = 0u;
                 if (w >= pw) {
@@ -660,6 +684,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                         if (diffs_before(nx) > diffs_before(32 * w + 31 - __clz(b))) f |= tail;
                     }
                     uint32_t inner = d & ~lead & ~tail;   // classes inside the word
+#pragma unroll 1
                     while (inner) {
                         const int q = __ffs(inner) - 1;
                         const uint32_t lo = 31 - __clz(b & lanes_below(q + 1)), up = b & (0xFFFFFFFEu << q);
@@ -689,6 +714,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 __syncthreads();
                 continue;
             }
+#pragma unroll 1
             for (int w = wa; w < wb; ++w) {
                 st.nzpre[w] = nzs;
                 if (w >= pw) nzs += __popc(st.touch[w] & st.flag[w]);
@@ -707,6 +733,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 return b ? (q & ~31) + __ffs(b) - 1 : (q >> 5) + 1 < wn ? st.next[(q >> 5) + 1] : n;
             };
             // ---- moved members listed, the others shifted to the end of their class
+#pragma unroll 1
             for (int q0 = (i2 & ~(G - 1)) + G * t; q0 < n; q0 += G * T) {
                 const int w = q0 >> 5, sh = q0 & 31;
                 uint32_t f = (st.flag[w] >> sh) & low_bits(min(G, n - q0));
@@ -742,6 +769,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
             // ---- the moved members in their new order
             if (r > 1) {
                 if (sc->nz_max <= kPanelCount) {   // four lanes count the members of e's class before e
+#pragma unroll 1
                     for (int e0 = warp * 8; e0 < m; e0 += NW * 8) {
                         const int e = min(e0 + (lane >> 2), m - 1);
                         const unsigned long long c = st.comp[e];
@@ -755,10 +783,13 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                     }
                 } else {
                     int p = 64;
+#pragma unroll 1
                     while (p < m) p <<= 1;
+#pragma unroll 1
                     for (int e = m + t; e < p; e += T) st.comp[e] = ~0ull;
                     __syncthreads();
                     panel_sort<T>(st.comp, p);
+#pragma unroll 1
                     for (int e = t; e < m; e += T) {
                         const unsigned long long c = st.comp[e];
                         const int s = (int)(c >> 44);
@@ -768,6 +799,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 __syncthreads();
             }
             // ---- back into perm, with the new boundaries (a warp's lanes share words: old ones are read first)
+#pragma unroll 1
             for (int c = (i2 & ~(32 * G - 1)) + warp * 32 * G; c < n; c += T * G) {
                 const int q0 = c + G * lane, w = q0 >> 5, sh = q0 & 31;
                 uint32_t f = q0 < n ? (st.flag[w] >> sh) & low_bits(min(G, n - q0)) : 0u;
@@ -815,6 +847,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
         if (ppos) {   // (a split class's members have moved: its starts' keys are looked up)
             constexpr int U = 4;   // words at once, so that their gathers overlap
             const bool split = sc->any != 0;
+#pragma unroll 1
             for (int w0 = (i2 >> 5) + warp; w0 < wn; w0 += U * NW) {
                 Id v[U];
                 uint32_t k[U], b[U];
