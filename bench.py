@@ -968,7 +968,7 @@ def run_gpu(args):
             per_launch = 1
         kernel = "lexbfs_dense_kernel" if wl == "dense16k" else "lexbfs_csr_kernel"
         if mcs:
-            kernel = "mcs_dense_kernel"
+            kernel = "mcs_panel_kernel"
         lex_gbs = lex_bytes / (lex_ms * 1e-3) / 1e9
         chk_gbs = chk_bytes / (chk_ms * 1e-3) / 1e9
         dom_share = prof["lexbfs_ms"] / max(1e-9, prof["lexbfs_ms"] + prof["check_ms"])

@@ -39,7 +39,7 @@
 // perfect-elimination check (Section 5.2).
 //
 // Measured on GB300 (whole test, one step per vertex -> panels): 65,536 vertices
-// of degree 21 122.3 -> 26.4 ms, 262,143 515 -> 126 ms, 5,000 8.0 -> 2.8 ms, 20,000
+// of degree 21 120.5 -> 25.8 ms, 262,143 506 -> 121 ms, 5,000 8.0 -> 2.8 ms, 20,000
 // of degree 5 28.0 -> 8.6 ms.  A panel of 30 pivots takes about 12 us: gathering
 // 2, the order 1.7, sorting 3, new classes 4.5, the front and barriers the rest;
 // all of it latency (barriers, dependent loads from L2, instruction fetch).

@@ -33,11 +33,12 @@
 // vertices on chordal, dense random, sparse random and tree inputs.
 //
 // Measured on GB300 (whole test; one step per vertex -> this): the pair of
-// n = 16,384 graphs at density 0.1 28.5 -> 4.36 ms (8.2 us per panel of 31),
-// G(10,000, 0.5) 49.7 -> 1.94 ms, n = 41,003 104.7 -> 34 ms, 4,096 graphs of
-// 16..2,048 vertices 3.77 -> 1.55 ms, one graph of 1,000 vertices 919 -> 193 us.
-// What bounds a panel is latency: the rows' L2 loads, the transpose's issue
-// slots, three CTA barriers and instruction fetch.
+// n = 16,384 graphs at density 0.1 28.3 -> 4.2 ms (7.7 us per panel of 31),
+// G(10,000, 0.5) 49.4 -> 1.85 ms, n = 41,003 104 -> 32.6 ms, 4,096 graphs of
+// 16..2,048 vertices 3.8 -> 1.47 ms, one graph of 1,000 vertices 913 -> 175 us.
+// What bounds a panel is latency and issue: the rows' L2 loads and their
+// transpose (a third), the passes over positions, the barriers, and instruction
+// fetch (code that runs once per panel is rolled where it can be).
 //
 // State: perm[] holds the vertices by position (numbered ones in front, then
 // class after class, ascending ids inside a class), and the class boundaries

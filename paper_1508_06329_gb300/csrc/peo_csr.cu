@@ -148,9 +148,10 @@ int csr_to_bits_launch(int n, const int64_t *row_ptr, const int32_t *col, uint32
 }
 
 bool csr_takes_dense_path(int n, int64_t nnz) {
-    // measured on GB300: a graph of average degree 21 at n = 65,536 runs 1.9 us per step on the
-    // CSR kernels against 9.6 on the dense ones; at degree ~500 and more the CSR search's
-    // CTA-wide long-row steps cost far more than a dense step (0.5 s against 9.5 s per graph)
+    // The CSR search's panels cost by the entries of 32 rows, the dense ones by n: on GB300 65,536
+    // vertices of degree 21 take 25.8 ms on the CSR kernels, 41,003 of degree 820 32.6 ms on the dense
+    // ones.  The line was drawn for the searches of one step per vertex (9.6 us a dense step at 65,536
+    // against 1.9 on CSR at degree 21, far more on CSR from degree 500 on).
     return n <= kCsrDenseMaxN && (n <= 4096 || (n > 0 && nnz >= 64 * (int64_t)n));
 }
 
