@@ -29,7 +29,7 @@
 // beat).  So the panels keep count of what they gained; when they have lost
 // kMcsPatience steps, they leave the rest to mcs_step_kernel.
 // n = 16,384 at density 0.1: 15.1 -> 6.8 ms, 9,000 at density 0.05 6.0 -> 3.0, a clique of 9,000 16.0 -> 8.4;
-// G(10,000, 1/2), which soon goes on in steps, 10.7 -> 10.9.
+// G(10,000, 1/2), which soon goes on in steps, 10.7 -> 11.1.
 #include <algorithm>
 
 #include "kernels.h"
