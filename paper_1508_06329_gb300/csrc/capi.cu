@@ -32,6 +32,7 @@ const char *cg_debug_array_name(unsigned code) {
         case kChkSplit: return "dense LexBFS split words";
         case kChkSort: return "dense LexBFS split sort";
         case kChkNumbered: return "dense LexBFS numbered mask";
+        case kChkPpos: return "dense LexBFS parents by position";
         case kChkCsrCls: return "CSR LexBFS cls";
         case kChkCsrNext: return "CSR LexBFS class next";
         case kChkCsrRec: return "CSR LexBFS class record";

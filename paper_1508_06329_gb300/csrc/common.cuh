@@ -141,7 +141,7 @@ __device__ __forceinline__ T *cg_arr(T *p, unsigned long long, unsigned) {
 
 // Array codes of the bounds-checking build (the high byte of the error word).
 enum : unsigned {
-    kChkCls = 1, kChkPerm, kChkKey, kChkSplit, kChkSort, kChkNumbered,
+    kChkCls = 1, kChkPerm, kChkKey, kChkSplit, kChkSort, kChkNumbered, kChkPpos,
     kChkCsrCls = 16, kChkCsrNext, kChkCsrRec, kChkCsrFree, kChkCsrSub, kChkCsrSkey, kChkCsrArena,
     kChkUnitMask = 40, kChkUnitPos, kChkUnitRow, kChkUnitGroup,
     kChkInjected = 255,

@@ -429,7 +429,9 @@ __device__ __forceinline__ void panel_write_mask(uint32_t *emask, int b, int n, 
 template <int STATE, int T>
 __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int n,
                               const PanelState<typename PanelId<STATE>::type> &st, PanelScalars *sc,
-                              int32_t *__restrict__ order, int32_t *__restrict__ pos, int32_t *ppos, uint32_t *emask) {
+                              int32_t *__restrict__ order, int32_t *__restrict__ pos, int32_t *ppos_out,
+                              uint32_t *emask) {
+    if (n <= 0) return;   // (ppos has no entry then: a batch packs the next graph's there)
     using Id = typename PanelId<STATE>::type;
     constexpr int NW = T / 32;
     constexpr unsigned kAll = 0xFFFFFFFFu;
@@ -441,6 +443,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
     constexpr int G = T >= 512 ? 8 : 1;
     const int t = threadIdx.x, lane = t & 31, warp = warp_index();
     const int wn = (n + 31) >> 5;
+    const auto ppos = cg_arr(ppos_out, n, kChkPpos);
 
 #pragma unroll 1
     for (int q = t; q < 32 * wn; q += T) st.perm[q] = (Id)q;   // positions past n too: they are read in eights
@@ -452,7 +455,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
         st.flag[w] = 0u;
         st.numbered[w] = 0u;
     }
-    if (t == 0 && ppos) ppos[0] = -1;
+    if (t == 0 && ppos_out) ppos[0] = -1;
     __syncthreads();
 
     int eb = 0;   // E_eb is to be written at the start of the next panel (0: none)
@@ -465,7 +468,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
             __funnelshift_r(st.start[i >> 5], (i >> 5) + 1 < wn ? st.start[(i >> 5) + 1] : 0u, i & 31) & low_bits(w2);
         const bool straddle = i + w2 < n && !((st.start[(i + w2) >> 5] >> ((i + w2) & 31)) & 1u);
         int cp = -1;   // warp 0: the classes' last adjacent pivots, requested early
-        if (warp == 0 && ppos && lane < w2) cp = __ldcg(ppos + i + lane);
+        if (warp == 0 && ppos_out && lane < w2) cp = __ldcg(&ppos[i + lane]);
         if (eb > 0) panel_write_mask<T>(emask, eb, n, st.numbered);
         reinterpret_cast<uint32_t *>(sc->row4)[lane] = 4u * (uint32_t)vk;
         __syncwarp();
@@ -514,7 +517,7 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                 if (i2 < n && !((st.start[i2 >> 5] >> (i2 & 31)) & 1u)) {
                     st.start[i2 >> 5] |= 1u << (i2 & 31);
                     set = i2;
-                    if (ppos) ppos[i2] = cpl;
+                    if (ppos_out) ppos[i2] = cpl;
                 }
                 sc->set_start = set;
                 sc->r = r;
@@ -816,9 +819,9 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
                     if (k != kp && !((bw >> (sh + e)) & 1u)) {
                         fresh |= 1u << e;
                         // the members that did not move keep the class's last adjacent pivot
-                        if (ppos && k == 0u) {
+                        if (ppos_out && k == 0u) {
                             const uint32_t le = bw & low_bits(sh + e + 1);
-                            ppos[q] = __ldcg(ppos + (le ? (w << 5) + 31 - __clz(le) : st.last[w - 1]));
+                            ppos[q] = __ldcg(&ppos[le ? (w << 5) + 31 - __clz(le) : st.last[w - 1]]);
                         }
                     }
                     kp = k;
@@ -842,10 +845,10 @@ __device__ void lexbfs_panels(const uint32_t *__restrict__ rows, int stride, int
             const int v = sc->piv[lane];
             order[i + lane] = v;
             if (pos) pos[v] = i + lane;
-            if (ppos) ppos[i + lane] = sc->par[lane];
+            if (ppos_out) ppos[i + lane] = sc->par[lane];
             if (eb == 0 || i + lane < 32 * eb) atomicOr(&st.numbered[v >> 5], 1u << (v & 31));
         }
-        if (ppos) {   // (a split class's members have moved: its starts' keys are looked up)
+        if (ppos_out) {   // (a split class's members have moved: its starts' keys are looked up)
             constexpr int U = 4;   // words at once, so that their gathers overlap
             const bool split = sc->any != 0;
 #pragma unroll 1
