@@ -569,16 +569,34 @@ struct Moved {
     const int32_t *row;
     int m;
     const uint32_t *bits;   // long row: bit k: k is the first of its class (null: not kept)
+    const int *last;        // and the last of these up to the end of a word
     __device__ __forceinline__ int cls(int k) const { return (int)(key[k] >> 32); }
     __device__ __forceinline__ int vertex(int k) const { return LONG ? row[key[k] & 0xFFFFFFFFu] : sh->y2[k]; }
     __device__ __forceinline__ bool first(int k) const {   // of its old class
-        return LONG ? k == 0 || cls(k - 1) != cls(k) : (sh->cstart[k >> 5] >> (k & 31)) & 1u;
+        if (LONG && !bits) return k == 0 || cls(k - 1) != cls(k);
+        return ((LONG ? bits : sh->cstart)[k >> 5] >> (k & 31)) & 1u;
+    }
+    __device__ __forceinline__ bool group_first(int k) const {   // of its new class
+        return LONG ? first(k) : (sh->gstart[k >> 5] >> (k & 31)) & 1u;
     }
     // the first index of k's new class; of its old one; the first index after its new one
     __device__ __forceinline__ int group_start(int k) const { return LONG ? key_start(k) : bit_at_or_before(sh->gstart, k); }
     __device__ __forceinline__ int class_start(int k) const { return LONG ? key_start(k) : bit_at_or_before(sh->cstart, k); }
     __device__ __forceinline__ int group_end(int k) const {
-        if (LONG && !bits) {
+        if (LONG && bits) {   // the first word beyond k's with another last start
+            int w = k >> 5, hi = (m - 1) >> 5;
+            const uint32_t b = bits[w] & (0xFFFFFFFEu << (k & 31));
+            if (b) return 32 * w + __ffs(b) - 1;
+            const int own = last[w];
+            if (last[hi] == own) return m;
+#pragma unroll 1
+            while (hi - w > 1) {
+                const int mid = (w + hi) >> 1;
+                if (last[mid] == own) w = mid; else hi = mid;
+            }
+            return 32 * hi + __ffs(bits[hi]) - 1;
+        }
+        if (LONG) {
             const int c = cls(k);
             int lo = k, st = 1;   // lo is in the class
 #pragma unroll 1
@@ -588,15 +606,17 @@ struct Moved {
                 if (lo + st < m && cls(lo + st) == c) lo += st;
             return lo + 1;
         }
-        const uint32_t *starts = LONG ? bits : sh->gstart;
         int w = k >> 5;
-        uint32_t b = starts[w] & (0xFFFFFFFEu << (k & 31));
+        uint32_t b = sh->gstart[w] & (0xFFFFFFFEu << (k & 31));
 #pragma unroll 1
-        while (!b && 32 * ++w < m) b = starts[w];
+        while (!b && 32 * ++w < m) b = sh->gstart[w];
         return b ? 32 * w + __ffs(b) - 1 : m;
     }
     __device__ __forceinline__ int key_start(int k) const {
-        if (bits) return bit_at_or_before(bits, k);
+        if (bits) {   // (bit 0 is set)
+            const uint32_t b = bits[k >> 5] & low_bits((k & 31) + 1);
+            return b ? (k & ~31) + 31 - __clz(b) : last[(k >> 5) - 1];
+        }
         const int c = cls(k);
         int hi = k, st = 1;
 #pragma unroll 1
@@ -623,7 +643,7 @@ __device__ __forceinline__ void move_ids(const CsrState &s, CsrShared *sh, const
                                          int *sub) {
 #pragma unroll 1
     for (int k = threadIdx.x; k < mv.m; k += kCsrThreads) {
-        if (mv.group_start(k) != k) continue;
+        if (!mv.group_first(k)) continue;
         const int c = mv.cls(k);
         const bool first = mv.first(k);
         const int4 rc = s.rec[c];
@@ -1054,11 +1074,13 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
         // nothing in the list but vertices that had no numbered neighbour: what the panel met goes to the front
         const bool to_front = !long_row && m > 0 && fl2 + m <= kFrontCap && sh->head_next == n &&
                               (int)(sh->key2[0] >> 32) == n;
-        const Moved<false> mv{sh, sh->key2, nullptr, m, nullptr};
+        const Moved<false> mv{sh, sh->key2, nullptr, m, nullptr, nullptr};
         uint32_t *lbits = reinterpret_cast<uint32_t *>(sh->y);   // y, y2 and sub
+        int *llast = reinterpret_cast<int *>(sh->key);           // key and key2
+        static_assert(sizeof(sh->key) + sizeof(sh->key2) >= 3 * kMaxEntries * sizeof(int), "a word of starts per int");
         const bool keep_bits = long_row && m <= 3 * 32 * kMaxEntries;
-        const Moved<true> ml{sh, lkey, g.col + f->beg[0], m, keep_bits ? lbits : nullptr};
-        if (keep_bits)
+        const Moved<true> ml{sh, lkey, g.col + f->beg[0], m, keep_bits ? lbits : nullptr, llast};
+        if (keep_bits) {
 #pragma unroll 1
             for (int k0 = 32 * warp; k0 < m; k0 += kCsrThreads) {
                 const int k = k0 + lane;
@@ -1066,6 +1088,32 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
                     __ballot_sync(kFull, k < m && (k == 0 || lkey[max(k - 1, 0)] >> 32 != lkey[k] >> 32));
                 if (lane == 0) lbits[k0 >> 5] = cb;
             }
+            __syncthreads();
+            // the last start up to each word's end, so that no member walks back through its class (a row of
+            // 65,000 members of one class: 6 ms by walking)
+            const int nw = (m + 31) >> 5, per = (nw + kCsrThreads - 1) / kCsrThreads;
+            const int a = min(t * per, nw), b = min(a + per, nw);
+            int own = -1;
+#pragma unroll 1
+            for (int w = a; w < b; ++w)
+                if (lbits[w]) own = 32 * w + 31 - __clz(lbits[w]);
+            int incl = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl = max(incl, u);
+            }
+            if (lane == 31) sh->scan[warp] = incl;
+            __syncthreads();
+            int at = __shfl_up_sync(kFull, incl, 1);
+            if (lane == 0) at = -1;
+            at = max(at, __reduce_max_sync(kFull, lane < warp ? sh->scan[lane] : -1));
+#pragma unroll 1
+            for (int w = a; w < b; ++w) {
+                if (lbits[w]) at = 32 * w + 31 - __clz(lbits[w]);
+                llast[w] = at;
+            }
+        }
         if (!long_row && !to_front)
 #pragma unroll 1
             for (int k0 = 32 * warp; k0 < m; k0 += kCsrThreads) {
