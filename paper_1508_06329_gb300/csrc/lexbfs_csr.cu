@@ -166,11 +166,6 @@ __global__ void csr_init_kernel(int *ws, int64_t n, int64_t max_deg, int32_t *pa
     }
 }
 
-// A barrier of some of the CTA's warps.
-__device__ __forceinline__ void named_barrier(int id, int threads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
 // Sorts the moved vertices key/y[0..m) by (key, y) into key2/y2, m <= kMaxEntries:
 // every warp sorts 32 in registers, then a vertex's rank is its place in its run
 // plus the vertices before it in every other run, found by bisection, two runs

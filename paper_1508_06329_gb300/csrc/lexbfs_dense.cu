@@ -44,11 +44,10 @@ __global__ void __launch_bounds__(T) lexbfs_dense_kernel(const DenseDesc *__rest
         const DenseDesc d = descs ? descs[gi] : single;
         const int n = d.n;
         prefetch_range_l2<T>(d.rows, (size_t)n * d.words * sizeof(uint32_t));
-        const auto st = panel_carve<STATE>(smem + kPanelScalarBytes,
-                                           STATE == kStateSmem ? nullptr : gstate + (size_t)blockIdx.x * gstate_stride,
-                                           n, cap);
-        lexbfs_panels<STATE, T>(d.rows, d.words, n, st, sc, order + d.obase, pos ? pos + d.vbase : nullptr,
-                                ppos ? ppos + d.vbase : nullptr, emask ? emask + d.ebase : nullptr);
+        lexbfs_panels<STATE, T>(d.rows, d.words, n, cap,
+                                STATE == kStateSmem ? nullptr : gstate + (size_t)blockIdx.x * gstate_stride,
+                                order + d.obase, pos ? pos + d.vbase : nullptr, ppos ? ppos + d.vbase : nullptr,
+                                emask ? emask + d.ebase : nullptr);
         __syncthreads();
         if (count == 1) break;
     }
