@@ -23,13 +23,13 @@
 //      ones) is a bound that at least 32 vertices reach, usually about 130,
 //      which are ranked by counting; when more than kMcsCand reach it, the
 //      bound is bisected.
-// A panel numbers about 31 vertices on dense chordal graphs, 10 on G(n, 1/2) and
-// fewer on sparse ones, and costs as much as kMcsWorth steps (13 us against 0.92
-// us a step at n = 16,384; below about 8,000 vertices steps are too cheap to
-// beat).  So the panels keep count of what they gained; when they have lost
-// kMcsPatience steps, they leave the rest to mcs_step_kernel.
-// n = 16,384 at density 0.1: 15.1 -> 6.8 ms, 9,000 at density 0.05 6.0 -> 3.0, a clique of 9,000 16.0 -> 8.4;
-// G(10,000, 1/2), which soon goes on in steps, 10.7 -> 11.1.
+// A panel numbers about 31 vertices on dense chordal graphs, 10 on G(n, 1/2) (5 to
+// 7 of the first ones) and fewer on sparse ones, and costs as much as kMcsWorth
+// steps (13 us against 0.92 us a step at n = 16,384; below about 8,000 vertices
+// steps are too cheap to beat).  So the panels keep count of what they gained; when
+// they have lost kMcsPatience steps, they leave the rest to mcs_step_kernel.
+// n = 16,384 at density 0.1: 15.1 -> 6.7 ms, 9,000 at density 0.05 6.0 -> 3.0, a clique of 9,000 16.0 -> 8.4;
+// G(n, p), which soon goes on in steps: G(15,000, 1/2) 17.4 -> 17.5, G(10,000, 1/2) 9.9 -> 10.1.
 #include <algorithm>
 
 #include "kernels.h"
@@ -47,7 +47,10 @@ constexpr int kMcsCand = 512;
 constexpr size_t kMcsSmemRows = 200 * 1024;     // dynamic shared memory limit for the row copy
 constexpr int kMcsPanelMin = 8192, kMcsPanelMax = 36608;   // keys and counts in shared memory
 constexpr int kMcsWorth = 20;                   // steps that cost as much as a panel (13 to 18 us)
-constexpr int kMcsPatience = 25;                // steps lost before the panels stop
+// The panels stop when they have lost this many steps (the first panel, which has no counts to go by, aside), or,
+// after many that paid, this many and kMcsCredit more.  The second panel of G(n, p) numbers 5 vertices, that of the
+// subtree-intersection graphs 10 to 32: one look is enough, and a panel of G(10,000, 1/2) costs 35 us.
+constexpr int kMcsPatience = 12, kMcsCredit = 63;
 
 // What the panels leave to the steps.
 struct alignas(16) McsLeft {
@@ -261,7 +264,7 @@ __global__ void __launch_bounds__(kMcsThreads, 1) mcs_panel_kernel(DenseDesc d, 
             }
         }
         i += r;
-        if (++panels > 2) credit = min(credit + r - kMcsWorth, 2 * kMcsPatience);   // (the first have few counts to go by)
+        if (++panels > 1) credit = min(credit + r - kMcsWorth, kMcsCredit);
         if (i >= n) break;
         __syncthreads();
         // ---- the next window: at least `need` vertices reach the bound
@@ -372,6 +375,9 @@ __global__ void __launch_bounds__(T) mcs_step_kernel(DenseDesc d, int32_t *__res
         uint32_t *numbered = reinterpret_cast<uint32_t *>(smem + label_bytes);
         const uint32_t *rows = d.rows;
         int stride = d.words;
+        // (kept from the compiler: with the parameter's own registers in the step's addresses G(8,000, 1/2) took 7.28
+        // ms instead of 7.11, G(15,000, 1/2) 18.0 instead of 17.6)
+        asm volatile("" : "+l"(rows), "+r"(stride));
         const size_t rows_off = (state_bytes + 15) & ~size_t(15);
         if (rows_off + (size_t)n * wn * 4 <= smem_bytes) {   // compact copy (stride wn) beside the counts
             uint32_t *rs = reinterpret_cast<uint32_t *>(smem + rows_off);
@@ -391,8 +397,14 @@ __global__ void __launch_bounds__(T) mcs_step_kernel(DenseDesc d, int32_t *__res
         if (left) {
             for (int v = t; v < n; v += T) label[v] = (uint16_t)max((int)left->cnt[v] - 1, 0);
             for (int w = t; w < wn; w += T) {
-                uint32_t m = 0u;
-                for (int b = 0; b < 32 && 32 * w + b < n; ++b) m |= (left->cnt[32 * w + b] ? 0u : 1u) << b;
+                uint32_t m = 0u;   // (count 0: numbered, or past the end)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint16_t c[8];
+                    panel_load8(&left->cnt[32 * w + 8 * q], c);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) m |= (c[e] ? 0u : 1u) << (8 * q + e);
+                }
                 numbered[w] = m;
             }
             __syncthreads();
