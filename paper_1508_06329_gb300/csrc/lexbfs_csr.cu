@@ -18,11 +18,17 @@
 //   3. the neighbours met, sorted by (class, label, id), leave their classes:
 //      each run of equal (class, label) becomes a new class, placed before the
 //      old one.
+// On narrow graphs (paths, matchings, small components, interval graphs of small
+// degree) the next vertex is known only after the one before, and a window numbers
+// two to ten.  When the windows do not pay, the front goes back to the list and warp
+// 0 takes pivots one by one, a lane per vertex that has met one (csr_steps); windows
+// are tried again from time to time.
 //
 // State.  A class is a segment of an arena of vertices, in id order; a member is
 // live while cls[] still names the class, so leaving a class costs one store.
 // New segments are cut from the arena's end; when it is full the live ones are
-// packed (7 n entries, so a packing follows at least 5 n moves).  Classes are in
+// packed (3 n entries and 4 for every one of the longest row, so a packing
+// follows at least 2 n moves).  Classes are in
 // a doubly linked list, top first; the next pointers of the first ids live in
 // shared memory, because following them is the one serial chain left.  The
 // class of the vertices without a numbered neighbour (id n) ends the list and
@@ -39,10 +45,13 @@
 // perfect-elimination check (Section 5.2).
 //
 // Measured on GB300 (whole test, one step per vertex -> panels): 65,536 vertices
-// of degree 21 120.5 -> 25.8 ms, 262,143 506 -> 121 ms, 5,000 8.0 -> 2.8 ms, 20,000
-// of degree 5 28.0 -> 8.6 ms.  A panel of 30 pivots takes about 12 us: gathering
+// of degree 21 120.5 -> 25.7 ms, 262,143 506 -> 122 ms, 5,000 8.0 -> 2.8 ms, 20,000
+// of degree 5 28.0 -> 8.5 ms.  A panel of 30 pivots takes about 12 us: gathering
 // 2, the order 1.7, sorting 3, new classes 4.5, the front and barriers the rest;
 // all of it latency (barriers, dependent loads from L2, instruction fetch).
+// Narrow, 65,536 vertices (windows alone in brackets): path 91 -> 53 ms (279),
+// matching 74 -> 40 (308), disjoint K4 70 -> 42 (164), K10 66 -> 51 (70), random
+// of degree 1 70 -> 37 (135).
 #include <algorithm>
 
 #include "kernels.h"
@@ -66,7 +75,10 @@ constexpr int kHashSize = 4096;        // at least kMaxEntries + kFrontCap
 constexpr int kFrontCap = 128;
 constexpr int kFrontLow = 64;          // the front is filled up to this many vertices beyond the window
 constexpr int kNextSmem = 30 * 1024;   // next pointers kept in shared memory
-constexpr int kScanStop = 128;         // a scan that has found a member looks at this many more slots
+// Windows give way to steps when they have numbered this many vertices less than kStepsBelow each: a window's panel
+// costs 8 to 12 us, a step 0.65 to 0.9.
+constexpr int kCsrStepsLost = 36;
+constexpr int kScanStop = 128;                // a scan that has found a member looks at this many more slots
 
 // State in the workspace.
 struct CsrState {
@@ -687,6 +699,254 @@ __device__ __forceinline__ void move_members(const CsrState &s, CsrShared *sh, c
     }
 }
 
+// The front's classes go back to the head of the list (warp 0).
+__device__ void front_to_list(const CsrState &s, CsrShared *sh, const CsrGraph &g, const Front *f) {
+    const int lane = threadIdx.x & 31, fl = sh->flen;
+    const int head = sh->head_next, ftop = sh->free_top;
+    const unsigned atop = sh->atop;
+    __syncwarp();
+    int before = 0;   // classes that start in the masks' earlier words
+#pragma unroll 1
+    for (int p0 = 0; p0 < fl; p0 += 32) {
+        const int p = p0 + lane;
+        const uint32_t starts = sh->fstart[p0 >> 5] & low_bits(fl - p0);
+        const int k = before + __popc(starts & low_bits(lane + 1)) - 1;
+        if (p < fl) {
+            const int id = s.freel[ftop - 1 - k], v = f->v[p];
+            s.arena[atop + p] = v;
+            s.cls[v] = id;
+            if (g.parent) g.parent[v] = f->par[p];
+            if ((starts >> lane) & 1u) {
+                int e = fl;   // the next class's start
+#pragma unroll 1
+                for (int w = p0 >> 5; 32 * w < fl; ++w) {
+                    const uint32_t b = sh->fstart[w] & (w == (p0 >> 5) ? 0xFFFFFFFEu << lane : kFull);
+                    if (b) {
+                        e = min(e, 32 * w + __ffs(b) - 1);
+                        break;
+                    }
+                }
+                const int next = e < fl ? s.freel[ftop - 2 - k] : head;
+                s.rec[id] = make_int4((int)(atop + p), (int)(atop + e), e - p, k > 0 ? s.freel[ftop - k] : kHead);
+                set_next(s, sh, g, id, next);
+                if (e == fl) s.rec[head].w = id;
+                if (k == 0) sh->head_next = id;
+            }
+        }
+        before += __popc(starts);
+        __syncwarp();
+    }
+    if (lane == 0) {
+        sh->free_top = ftop - before;
+        sh->atop = atop + (unsigned)fl;
+        sh->flen = 0;
+    }
+    if (lane < kFrontCap / 32) sh->fstart[lane] = 0u;
+    __syncwarp();
+}
+
+// Panels of up to 32 pivots one by one, by warp 0 alone, on the list (the front is
+// empty): for narrow graphs, whose next vertices the window does not hold.  A lane
+// per vertex that has met a pivot and is not numbered yet: its class, its label in
+// this panel, its row.  A step reads the pivot's row (at most 32 entries) and the
+// classes and rows of the neighbours (two dependent L2 loads); the next pivot is
+// the lane of the class at hand with the largest label, or that class's first
+// member that has not been met.  At the panel's end the lanes move to their new
+// classes as after a window.  Ends early before a pivot with a longer row or one
+// that meets more vertices than lanes are free.  Leaves the number of pivots in sh->r.
+__device__ void csr_steps(const CsrState &s, CsrShared *sh, const CsrGraph &g, int i, int32_t *__restrict__ order,
+                          int32_t *__restrict__ pos, int panels) {
+    const int n = g.n, lane = threadIdx.x & 31;
+    int total = 0;
+    bool stop = false;
+#pragma unroll 1
+    for (; panels > 0 && !stop && i + total < n && s.cap - sh->atop >= 32u; --panels) {
+        int y = -1, cy = -1, dy = 0;    // the lane's vertex, its class, its row
+        int64_t by = 0;
+        uint32_t ky = 0u;               // its label in pivot order, the first pivot highest
+        int c = sh->head_next, z = 0;   // the class at hand, its live members
+        unsigned q = 0u, end = 0u;      // its slots from q on
+        int mv = -1, md = 0;            // the lane's member in q .. q + 31 (live, not met when it was looked at), its row
+        int64_t mb = 0;
+        auto members = [&]() {
+            const unsigned e = q + lane;
+            mv = e < end ? (c == n ? (int)e : s.arena[e]) : -1;
+            const int x = max(mv, 0);
+            const int cl = s.cls[x];
+            mb = g.row_ptr[x];
+            md = (int)(g.row_ptr[x + 1] - mb);
+            if (cl != c) mv = -1;
+        };
+        auto enter = [&]() {
+            const int4 rc = c == n ? make_int4(sh->unl_cur, n, sh->unl_size, 0) : s.rec[c];
+            q = (unsigned)rc.x;
+            end = (unsigned)rc.y;
+            z = rc.z;
+            members();
+        };
+        auto leave = [&]() {   // the class at hand is used up
+            const int nx = get_next(s, sh, g, c);
+            __syncwarp();
+            if (lane == 0) {
+                s.freel[sh->free_top++] = c;
+                sh->head_next = nx;
+                s.rec[nx].w = kHead;
+            }
+            __syncwarp();
+            c = nx;
+        };
+        enter();
+        int r = 0;
+#pragma unroll 1
+        for (;;) {
+            // ---- the next pivot
+            int x = -1, deg = 0;
+            int64_t beg = 0;
+            uint32_t label;
+#pragma unroll 1
+            for (;;) {
+                label = __reduce_max_sync(kFull, y >= 0 && cy == c ? ky : 0u);
+                if (label) {
+                    x = (int)__reduce_min_sync(kFull, y >= 0 && cy == c && ky == label ? (unsigned)y : kNoVertex);
+                    const int l = __ffs(__ballot_sync(kFull, y == x)) - 1;
+                    beg = __shfl_sync(kFull, by, l);
+                    deg = __shfl_sync(kFull, dy, l);
+                    break;
+                }
+                uint32_t ok = z > 0 ? __ballot_sync(kFull, mv >= 0) : 0u;
+#pragma unroll 1
+                while (ok) {
+                    const int l = __ffs(ok) - 1, v = __shfl_sync(kFull, mv, l);
+                    if (!__ballot_sync(kFull, y == v)) {
+                        x = v;
+                        beg = __shfl_sync(kFull, mb, l);
+                        deg = __shfl_sync(kFull, md, l);
+                        break;
+                    }
+                    if (lane == l) mv = -1;   // met
+                    ok &= ok - 1u;
+                }
+                if (ok) break;
+                if (z > 0 && q + 32 < end) {
+                    q += 32;
+                    members();
+                    continue;
+                }
+                if (c == n) break;   // (not on a well-formed graph)
+                leave();
+                enter();
+            }
+            // ---- its row
+            if (x < 0 || deg > 32) {
+                stop = true;
+                break;
+            }
+            const int w = lane < deg ? g.col[beg + lane] : -1, wx = max(w, 0);
+            const int cw = s.cls[wx];
+            const int64_t bw = g.row_ptr[wx];
+            const int dw = (int)(g.row_ptr[wx + 1] - bw);
+            bool adj = false, known = w < 0;
+#pragma unroll 1
+            for (int k = 0; k < deg; ++k) {
+                const bool is = y == __shfl_sync(kFull, w, k);
+                adj |= is;
+                if (__ballot_sync(kFull, is) && lane == k) known = true;
+            }
+            const bool fresh = !known && cw != kNumberedCls;
+            const uint32_t met = __ballot_sync(kFull, fresh), room = __ballot_sync(kFull, y < 0 || y == x);
+            if (__popc(met) > __popc(room)) {
+                stop = true;
+                break;
+            }
+            if (lane == 0) {
+                sh->piv[r] = x;
+                sh->scan[r] = label ? sh->piv[32 - __ffs((int)label)] : -2;   // (-2: what met it before this panel)
+                s.cls[x] = kNumberedCls;
+            }
+            if (y == x) y = -1;
+            if (mv == x) mv = -1;
+            --z;
+            const uint32_t bit = 0x80000000u >> r;
+            if (y >= 0 && adj) ky |= bit;
+            if (fresh) {
+                const int k = __popc(met & lanes_below(lane));
+                sh->y[k] = w;
+                sh->sub[k] = cw;
+                sh->key[k] = (unsigned long long)bw;
+                sh->key2[k] = (unsigned long long)(unsigned)dw;
+            }
+            __syncwarp();
+            const int k = __popc(room & lanes_below(lane));
+            if (((room >> lane) & 1u) && k < __popc(met)) {
+                y = sh->y[k];
+                cy = sh->sub[k];
+                by = (int64_t)sh->key[k];
+                dy = (int)sh->key2[k];
+                ky = bit;
+            }
+            __syncwarp();
+            ++r;
+            if (r == 32 || i + total + r == n) break;
+        }
+        // ---- what is left of the class at hand; the results
+        if (c == n) {
+            if (lane == 0) {
+                sh->unl_cur = (int)q;
+                sh->unl_size = z;
+            }
+        } else if (z == 0) {
+            leave();
+        } else if (lane == 0) {
+            s.rec[c].x = (int)q;
+            s.rec[c].z = z;
+        }
+        if (lane < r) {
+            const int v = sh->piv[lane], p = sh->scan[lane];
+            order[i + total + lane] = v;
+            if (pos) pos[v] = i + total + lane;
+            if (g.parent && p != -2) g.parent[v] = p;
+        }
+        __syncwarp();
+        // ---- the vertices met, by (class, label, id), to their new classes
+        const uint32_t on = __ballot_sync(kFull, y >= 0);
+        const int m = __popc(on);
+        if (m > 0) {
+            const unsigned long long mine = (unsigned long long)(unsigned)cy << 32 | (unsigned)~ky;
+            int rank = 0;
+#pragma unroll 1
+            for (uint32_t b = on; b; b &= b - 1u) {
+                const int l = __ffs(b) - 1;
+                const unsigned long long o = __shfl_sync(kFull, mine, l);
+                const int oy = __shfl_sync(kFull, y, l);
+                rank += o < mine || (o == mine && oy < y) ? 1 : 0;
+            }
+            if (y >= 0) {
+                sh->key2[rank] = mine;
+                sh->y2[rank] = y;
+            }
+            __syncwarp();
+            const unsigned long long o = lane < m ? sh->key2[lane] : 0ull, po = lane > 0 && lane < m ? sh->key2[lane - 1] : 0ull;
+            const uint32_t gb = __ballot_sync(kFull, lane < m && (lane == 0 || o != po));
+            const uint32_t cb = __ballot_sync(kFull, lane < m && (lane == 0 || o >> 32 != po >> 32));
+            if (lane == 0) {
+                sh->gstart[0] = gb;
+                sh->cstart[0] = cb;
+            }
+            __syncwarp();
+            const Moved<false> moved{sh, sh->key2, nullptr, m, nullptr, nullptr};
+            move_ids(s, sh, g, moved, sh->sub);
+            __syncwarp();
+            move_members(s, sh, g, moved, sh->sub, sh->atop);
+            __syncwarp();
+            if (lane == 0) sh->atop += (unsigned)m;
+            __syncwarp();
+        }
+        total += r;
+    }
+    if (lane == 0) sh->r = total;
+    __syncwarp();
+}
+
 __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_t max_deg, CsrGraph g, int64_t nnz,
                                                                  int32_t *__restrict__ order, int32_t *__restrict__ pos) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -726,8 +986,32 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
     int cur = 0;   // the front at hand
     const int fp = t - (kCsrThreads - kFrontCap);   // the last threads: position in the front
     const bool front_warp = warp >= (kCsrThreads - kFrontCap) / 32;
+    // pivots that windows have fallen short of kStepsBelow each; panels of steps that follow the next time
+    int lost = 0, span = 1;
     while (i < n) {
         Front *f = &sh->front[cur], *nf = &sh->front[cur ^ 1];
+        if (lost > kCsrStepsLost) {
+            const bool pack = s.cap - sh->atop < (unsigned)(kFrontCap + 32 * span);
+            __syncthreads();   // everyone has read the arena's end
+            if (pack) arena_pack(s, sh, g);
+            if (warp == 0) {
+                const bool room = s.cap - sh->atop >= (unsigned)kFrontCap;
+                __syncwarp();
+                if (lane == 0) sh->r = 0;
+                if (room) {
+                    front_to_list(s, sh, g, f);
+                    csr_steps(s, sh, g, i, order, pos, span);
+                }
+            }
+            __syncthreads();
+            const int r = sh->r;
+            i += r;
+            // the next window that does not pay is the last one, unless the steps did not pay either
+            lost = r < kStepsBelow ? 0 : kCsrStepsLost;
+            span = min(2 * span, kStepsMost);
+            __syncthreads();
+            continue;
+        }
         if (sh->flen == 0) {
             __syncthreads();
             if (warp == 0) front_fill(s, sh, g, f, 0, kFrontLow);
@@ -1193,6 +1477,8 @@ __global__ void __launch_bounds__(kCsrThreads) lexbfs_csr_kernel(int *ws, int64_
                 }
             }
         }
+        if (!long_row) lost = max(lost + kStepsBelow - r, 0);
+        if (r >= kStepsBelow) span = 1;
         i += r;
         cur ^= 1;
         __syncthreads();
