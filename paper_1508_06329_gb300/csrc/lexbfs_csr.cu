@@ -323,7 +323,7 @@ __device__ const unsigned long long *sort_long_row(CsrShared *sh, const int *kep
     uint32_t(*hist)[256] = reinterpret_cast<uint32_t(*)[256]>(sh->key);   // [NW][256]: key and key2
     unsigned long long *src = b2, *dst = b1;
 #pragma unroll 1
-    for (int shift = 0; shift == 0 || ((n - 1) >> shift) > 0; shift += 8) {
+    for (int shift = 0; shift == 0 || (shift < 32 && ((n - 1) >> shift) > 0); shift += 8) {
         const int len = shift ? m : d, part = (len + kCsrThreads - 1) / kCsrThreads * 32;
         const int lo = min(warp * part, len), hi = min(lo + part, len);
         auto load = [&](int k) -> unsigned long long {   // ~0: none
