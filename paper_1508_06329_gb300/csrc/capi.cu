@@ -41,7 +41,6 @@ const char *cg_debug_array_name(unsigned code) {
         case kChkCsrSkey: return "CSR LexBFS long-row keys";
         case kChkCsrArena: return "CSR LexBFS arena";
         case kChkUnitMask: return "check earlier-than mask";
-        case kChkUnitPos: return "check pos gather";
         case kChkUnitGroup: return "check order / parent value";
         case kChkInjected: return "injected test entry";
         default: return "unknown array";
@@ -388,8 +387,8 @@ int run_single_dense(cg_context *ctx, const cg_dense *g, int32_t *order_out, int
         if (!res) return CG_OK;
         PhaseTimer pt(ctx, &ctx->ev_check, stream);
         ctx->launches += 1;
-        return peo_dense_launch(nullptr, d, 1, nullptr, 0, order, pos, ppos, true, key, ctx->num_sms, stream,
-                                nullptr, 0, false, res);
+        return peo_dense_launch(nullptr, d, 1, nullptr, 0, order, pos, ppos, key, ctx->num_sms, stream, nullptr, 0,
+                                res);
     }
     // with a result wanted, the search also records the parents of its pivots
     // by position (one store per step) and initialises the check's keys
@@ -727,8 +726,8 @@ int cg_peo_check_dense(cg_context *ctx, const cg_dense *g, const int32_t *order,
     if (n > 0) CG_CUDA_TRY(cudaMemsetAsync(pos, 0xFF, sizeof(int32_t) * (size_t)n, stream));
     if ((rc = invert_order_launch(nullptr, d, 1, nullptr, n, order, pos, ctx->num_sms, stream))) return rc;
     ctx->launches += n > 0 ? 3 : 1;
-    return peo_dense_launch(nullptr, d, 1, nullptr, n, order, pos, par, false, key, ctx->num_sms, stream,
-                            at<uint32_t>(ctx, o_emask), n, false, res);
+    return peo_dense_launch(nullptr, d, 1, nullptr, n, order, pos, par, key, ctx->num_sms, stream,
+                            at<uint32_t>(ctx, o_emask), n, res);
 }
 
 int cg_chordal_test_dense_host(cg_context *ctx, int32_t n, int32_t words_per_row, const uint32_t *host_rows,
@@ -787,8 +786,8 @@ int run_mcs_dense(cg_context *ctx, const cg_dense *g, int32_t *order_out, int32_
     PhaseTimer pt(ctx, &ctx->ev_check, stream);
     unsigned long long *key = at<unsigned long long>(ctx, o_key);
     ctx->launches += n > 0 ? 2 : 1;
-    return peo_dense_launch(nullptr, d, 1, nullptr, n, order, pos, parent, false, key, ctx->num_sms, stream,
-                            at<uint32_t>(ctx, o_emask), n, false, res);
+    return peo_dense_launch(nullptr, d, 1, nullptr, n, order, pos, parent, key, ctx->num_sms, stream,
+                            at<uint32_t>(ctx, o_emask), n, res);
 }
 }  // namespace
 

@@ -148,12 +148,9 @@ __device__ __forceinline__ T *cg_arr(T *p, unsigned long long, unsigned) {
 enum : unsigned {
     kChkCls = 1, kChkPerm, kChkKey, kChkSplit, kChkSort, kChkNumbered, kChkPpos,
     kChkCsrCls = 16, kChkCsrNext, kChkCsrRec, kChkCsrFree, kChkCsrSub, kChkCsrSkey, kChkCsrArena,
-    kChkUnitMask = 40, kChkUnitPos, kChkUnitRow, kChkUnitGroup,
+    kChkUnitMask = 40, kChkUnitGroup,
     kChkInjected = 255,
 };
-
-// Parent value meaning "not known yet": the dense check finds it.
-constexpr int kParentUnresolved = -2;
 
 // Per-graph descriptor as the kernels see it (device memory).
 struct DenseDesc {

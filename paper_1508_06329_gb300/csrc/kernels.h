@@ -42,39 +42,37 @@ int debug_inject(unsigned code);
 
 // ---- dense perfect-elimination check (peo_dense.cu)
 // keys: device u64[count], set to ~0 by the launcher.
-// parent_known: parent[] already holds p(v) (from the search); otherwise the
-// kernel computes it from the rows and writes it.
+// parent: receives p(v) by vertex.
 // emask: workspace for the graphs' earlier-than masks (earlier_mask_words(n)
 // words at each desc's ebase; n_max = the largest n), or null for the
-// gather-based check.  prefilled (with masks, parent_known false): parent
-// already holds p(v) or kParentUnresolved for each v (from the search).
+// gather-based check.
 // res: when given, the results are written too (keys then needs count + 1
 // entries: the last counts the check's finished blocks); otherwise the
 // caller runs finalize_launch.
 int peo_dense_launch(const DenseDesc *descs, DenseDesc single, int count, const int64_t *voff, int64_t total,
-                     const int32_t *order, const int32_t *pos, int32_t *parent, bool parent_known,
-                     unsigned long long *keys, int num_sms, cudaStream_t stream, uint32_t *emask = nullptr,
-                     int n_max = 0, bool prefilled = false, cg_result *res = nullptr);
+                     const int32_t *order, const int32_t *pos, int32_t *parent, unsigned long long *keys,
+                     int num_sms, cudaStream_t stream, uint32_t *emask = nullptr, int n_max = 0,
+                     cg_result *res = nullptr);
 int64_t earlier_mask_words(int n);
 
-// The check of orders the dense LexBFS produced under kParentPivots (parents
-// by position in ppos, keys initialised by the search), in one launch: one
-// block per group of 32 positions (grid ceil(n_max / 32) x count) builds E_b
-// in shared memory from pos, resolves the group's open parents (stored back
-// into ppos) and checks its positions; its last block writes res.  vec when
+// The check of orders the dense LexBFS produced (exact parents by position in
+// ppos, keys initialised by the search), in one launch: one block per group of
+// 32 positions (grid ceil(n_max / 32) x count) builds E_b in shared memory from
+// pos and checks its positions; its last block writes res.  vec when
 // every graph passes peo_rows_vec_ok (rows 16-byte aligned, words_per_row a
 // multiple of 4: 128-bit row loads).  A result with chordal = -1 reports a
 // check that could not complete (an order or parent value outside 0..n-1).
 bool peo_rows_vec_ok(const DenseDesc &d);
 int peo_unit_launch(const DenseDesc *descs, DenseDesc single, int count, int n_max, bool vec, const int32_t *order,
-                    const int32_t *pos, int32_t *ppos, unsigned long long *keys, cg_result *res, cudaStream_t stream);
+                    const int32_t *pos, const int32_t *ppos, unsigned long long *keys, cg_result *res,
+                    cudaStream_t stream);
 // The same check with the rows staged in shared memory: persistent blocks
 // stage runs of 16 or 32 positions (their rows, the rows of the positions
 // just before, and E_b, which the search wrote: lexbfs_dense_launch's emask)
-// with bulk copies into two alternating buffers and test row_v & ~row_p & E_b
-// there.  Needs peo_stage_ok for every graph (rows suited to bulk copies,
-// n <= kStageMaxN), exact parents in ppos (the search's cpar) and the masks
-// at each desc's ebase.
+// with 16-byte asynchronous copies into two alternating buffers and test
+// row_v & ~row_p & E_b there.  Needs peo_stage_ok for every graph (rows suited to
+// those copies, n <= kStageMaxN), exact parents in ppos and the masks at each
+// desc's ebase.
 constexpr int kStageMaxN = 49152;
 bool peo_stage_ok(const DenseDesc &d);
 int peo_stage_launch(const DenseDesc *descs, DenseDesc single, int count, int n_max, const int32_t *order,

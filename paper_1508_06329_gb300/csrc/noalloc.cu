@@ -115,8 +115,7 @@ extern "C" int cg_chordal_test_dense_noalloc(const cg_dense *g, cg_result *res, 
     d.vbase = 0;
     d.obase = 0;
     if (n == 0)
-        return peo_dense_launch(nullptr, d, 1, nullptr, 0, ord, pos, ppos, true, key, num_sms, stream, nullptr, 0,
-                                false, res);
+        return peo_dense_launch(nullptr, d, 1, nullptr, 0, ord, pos, ppos, key, num_sms, stream, nullptr, 0, res);
     // the search sets the witness key to its "no violation" value
     if ((rc = lexbfs_dense_launch(plan, nullptr, d, 1, 1, ord, pos, ppos, nullptr, counter, stream, key))) return rc;
     return peo_unit_launch(nullptr, d, 1, n, peo_rows_vec_ok(d), ord, pos, ppos, key, res, stream);

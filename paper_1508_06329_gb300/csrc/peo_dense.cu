@@ -20,8 +20,7 @@
 // then streams row v, row p(v) and E_b (restricting to earlier vertices is a
 // word-wise AND, no pos gathers) and finds the remaining parents by probing
 // groups of 32 positions and a binary search over the masks.  Without masks
-// (the fixed-scratch entry point) p(v) comes from the caller or from pos
-// gathers over row v.
+// p(v) comes from pos gathers over row v.
 // The first violation in order is found by an atomicMin over the 64-bit
 // key (pos(v) << 32 | u), u being the lowest id of bad(v); the finalize
 // kernel turns each graph's key into (chordal, v, p, u).
@@ -42,6 +41,7 @@ constexpr int kRC = 8;    // row words per lane held in registers (256 words = 8
 // emask + ebase, row b = E_b.
 constexpr int kMaskRows = 8;          // rows b per mask tile
 constexpr int kScan = 32;             // positions a prep thread scans for p(v)
+constexpr int kParentUnresolved = -2; // p(v) lies before these: the check's warp finds it
 
 // (chordal, v, p, u) from a graph's key (pos(v*) << 32 | u*, or ~0 when chordal).
 __device__ __forceinline__ void write_result(const DenseDesc &d, unsigned long long k, const int32_t *order,
@@ -94,7 +94,6 @@ __device__ __forceinline__ bool has_bit(const uint32_t *__restrict__ row, int u)
 // p(v) is found by probing the order backwards from pos(v) in groups of 32
 // (after kProbe groups without a neighbour, a binary search over the masks
 // finds the last group that holds one).
-template <bool PARENT_KNOWN>
 __global__ void __launch_bounds__(kPeoThreads, 4) peo_dense_kernel(const DenseDesc *__restrict__ descs,
                                                                 DenseDesc single, int count,
                                                                 const int64_t *__restrict__ voff, int64_t total,
@@ -149,47 +148,42 @@ __global__ void __launch_bounds__(kPeoThreads, 4) peo_dense_kernel(const DenseDe
             xin = (unsigned)ux < (unsigned)d.n && has_bit(rv, ux);
         }
         int p;
-        if (PARENT_KNOWN || E) {
-            // known, or found by peo_prep_kernel's scan of the last kScan positions
-            p = __ldg(parent + d.vbase + v);
-        }
-        if (!PARENT_KNOWN) {
-            if (E) {
-                if (p == kParentUnresolved) {   // warp-wide: groups of 32 positions, then the masks
-                    p = -1;
-                    int c = (pv >> 5) - 1;
-                    for (int r = 0; c >= 0 && r < kProbe; --c, ++r) {
-                        const int u = __ldg(ord_g + c * 32 + lane);   // c * 32 + 31 < pos(v)
-                        const unsigned hit = __ballot_sync(0xFFFFFFFFu, (unsigned)u < (unsigned)d.n && has_bit(rv, u));
-                        if (hit) {
-                            p = __shfl_sync(0xFFFFFFFFu, u, 31 - __clz(hit));
-                            break;
-                        }
+        if (E) {
+            p = __ldg(parent + d.vbase + v);   // found by peo_prep_kernel's scan of the last kScan positions
+            if (p == kParentUnresolved) {   // warp-wide: groups of 32 positions, then the masks
+                p = -1;
+                int c = (pv >> 5) - 1;
+                for (int r = 0; c >= 0 && r < kProbe; --c, ++r) {
+                    const int u = __ldg(ord_g + c * 32 + lane);   // c * 32 + 31 < pos(v)
+                    const unsigned hit = __ballot_sync(0xFFFFFFFFu, (unsigned)u < (unsigned)d.n && has_bit(rv, u));
+                    if (hit) {
+                        p = __shfl_sync(0xFFFFFFFFu, u, 31 - __clz(hit));
+                        break;
                     }
-                    if (p < 0 && c >= 0) {
-                        // groups 0..c remain: F(g) = |row_v ∩ E_g| is nondecreasing in g; the
-                        // parent's group is the last g <= c with F(g) < F(c + 1)
-                        const int total = count_in(rv, emask + d.ebase + (size_t)(c + 1) * es, wn, lane);
-                        if (total > 0) {
-                            int lo = 0, hi = c + 1;   // F(lo) < total = F(hi)
-                            while (hi - lo > 1) {
-                                const int mid = (lo + hi) >> 1;
-                                if (count_in(rv, emask + d.ebase + (size_t)mid * es, wn, lane) == total) hi = mid;
-                                else lo = mid;
-                            }
-                            const int u = __ldg(ord_g + lo * 32 + lane);
-                            const unsigned hit =
-                                __ballot_sync(0xFFFFFFFFu, (unsigned)u < (unsigned)d.n && has_bit(rv, u));
-                            if (hit) p = __shfl_sync(0xFFFFFFFFu, u, 31 - __clz(hit));
-                        }
-                    }
-                    if (lane == 0) parent[d.vbase + v] = p;
                 }
-            } else {
-                const int best = parent_by_gather(rv, wn, lastmask, pos_g, pv, lane);
-                p = best >= 0 ? __ldg(ord_g + best) : -1;
+                if (p < 0 && c >= 0) {
+                    // groups 0..c remain: F(g) = |row_v ∩ E_g| is nondecreasing in g; the
+                    // parent's group is the last g <= c with F(g) < F(c + 1)
+                    const int total = count_in(rv, emask + d.ebase + (size_t)(c + 1) * es, wn, lane);
+                    if (total > 0) {
+                        int lo = 0, hi = c + 1;   // F(lo) < total = F(hi)
+                        while (hi - lo > 1) {
+                            const int mid = (lo + hi) >> 1;
+                            if (count_in(rv, emask + d.ebase + (size_t)mid * es, wn, lane) == total) hi = mid;
+                            else lo = mid;
+                        }
+                        const int u = __ldg(ord_g + lo * 32 + lane);
+                        const unsigned hit =
+                            __ballot_sync(0xFFFFFFFFu, (unsigned)u < (unsigned)d.n && has_bit(rv, u));
+                        if (hit) p = __shfl_sync(0xFFFFFFFFu, u, 31 - __clz(hit));
+                    }
+                }
                 if (lane == 0) parent[d.vbase + v] = p;
             }
+        } else {
+            const int best = parent_by_gather(rv, wn, lastmask, pos_g, pv, lane);
+            p = best >= 0 ? __ldg(ord_g + best) : -1;
+            if (lane == 0) parent[d.vbase + v] = p;
         }
         if (p < 0 || p >= d.n) continue;
 
@@ -305,17 +299,14 @@ __device__ void build_mask_tiles(const DenseDesc &d, const int32_t *__restrict__
 // The check's preparation, one launch per bucket of graphs (blockIdx.y =
 // graph): blocks [0, mask_blocks) build E_b, one warp per tile of 32 words w
 // (a lane per word, holding the position groups pos(u) / 32 of its 32
-// vertices) by kMaskRows rows b, so the stores of a row are coalesced; with
-// PARENTS, the other blocks give each vertex v whose parent is not known yet
-// (all of them, or with prefilled those marked kParentUnresolved) a thread
-// that scans the kScan positions before pos(v), 8 independent probes at a
-// time, for the latest neighbour: p(v), -1 (none exists) or kParentUnresolved
-// (left to the check's warp).
-template <bool PARENTS>
+// vertices) by kMaskRows rows b, so the stores of a row are coalesced; the other
+// blocks give each vertex v a thread that scans the kScan positions before pos(v),
+// 8 independent probes at a time, for the latest neighbour: p(v), -1 (none exists)
+// or kParentUnresolved (left to the check's warp).
 __global__ void peo_prep_kernel(const DenseDesc *__restrict__ descs, DenseDesc single,
                                 const int32_t *__restrict__ order, const int32_t *__restrict__ pos,
                                 int32_t *__restrict__ parent, uint32_t *__restrict__ emask, int mask_blocks,
-                                bool prefilled, unsigned long long *__restrict__ keys) {
+                                unsigned long long *__restrict__ keys) {
     if (keys && blockIdx.x == 0 && threadIdx.x == 0) {   // "no violation" key, and the check's block counter
         keys[blockIdx.y] = ~0ull;
         if (blockIdx.y == 0) keys[gridDim.y] = 0ull;
@@ -327,11 +318,9 @@ __global__ void peo_prep_kernel(const DenseDesc *__restrict__ descs, DenseDesc s
         build_mask_tiles(d, pos_g, emask, mask_blocks);
         return;
     }
-    if (!PARENTS) return;
     const int32_t *ord_g = order + d.obase;
     const int stride = (gridDim.x - mask_blocks) * blockDim.x;
     for (int v = (blockIdx.x - mask_blocks) * blockDim.x + threadIdx.x; v < n; v += stride) {
-        if (prefilled && parent[d.vbase + v] != kParentUnresolved) continue;
         const int pv = __ldg(pos_g + v);
         if (pv < 0 || pv >= n) continue;   // skipped by the check as well
         const uint32_t *rv = d.rows + (size_t)v * d.words;
@@ -419,30 +408,23 @@ __device__ __forceinline__ uint4 ldg4(const uint32_t *p) { return __ldg(reinterp
 //   1. it builds E_b, the vertices numbered before position 32 b, in shared
 //      memory from pos (a word per thread and pass: the pos of its 32
 //      vertices against 32 b; pos is small enough to stay in L1);
-//   2. it resolves the parents the search left open in the group
-//      (kParentUnresolved: pivots taken from the class after the top one),
-//      one vertex per warp: p(v) is the earlier neighbour with the largest
-//      position, from pos gathered over row v (row words loaded first, then
-//      one predicated load per bit position);
-//   3. each warp checks four of the positions: the lowest bit of row_v &
+//   2. each warp checks four of the positions: the lowest bit of row_v &
 //      ~row_p & E_b other than p (row v and row p loaded 128 bits per lane,
 //      E_b read from shared memory), plus the group's own earlier positions
 //      one per lane; the first violation in order is kept by an atomicMin of
 //      (pos(v) << 32 | u) and the last block writes the results.
 constexpr int kUnitThreads = 256;
 constexpr int kUnitWarps = kUnitThreads / 32;
-constexpr int kGatherWords = 16;   // row words per lane held at once by a gathering warp
 
 template <bool VEC>
 __global__ void __launch_bounds__(kUnitThreads) peo_unit_kernel(const DenseDesc *__restrict__ descs, DenseDesc single,
                                                                 int count, const int32_t *__restrict__ order,
                                                                 const int32_t *__restrict__ pos,
-                                                                int32_t *__restrict__ ppos,
+                                                                const int32_t *__restrict__ ppos,
                                                                 unsigned long long *__restrict__ keys,
                                                                 cg_result *__restrict__ res) {
     extern __shared__ __align__(16) uint32_t sE[];   // mask_stride(n) words
     __shared__ int s_v[32], s_p[32];
-    __shared__ unsigned s_open;
     __shared__ bool s_last;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int gi = blockIdx.y;
@@ -454,12 +436,11 @@ __global__ void __launch_bounds__(kUnitThreads) peo_unit_kernel(const DenseDesc 
         const uint32_t lastmask = (n & 31) ? ((1u << (n & 31)) - 1u) : 0xFFFFFFFFu;
         const int32_t *pos_g = pos + d.vbase;
         const int32_t *ord_g = order + d.obase;
-        int32_t *pp_g = ppos + d.vbase;
+        const int32_t *pp_g = ppos + d.vbase;
         if (warp == 0) {   // the group's vertices and parents (values outside 0..n-1 are reported)
             int v = g0 + lane < n ? __ldg(ord_g + g0 + lane) : -1;
             int p = g0 + lane < n ? __ldg(pp_g + g0 + lane) : -1;
-            const bool bad =
-                g0 + lane < n && ((unsigned)v >= (unsigned)n || p >= n || (p < -1 && p != kParentUnresolved));
+            const bool bad = g0 + lane < n && ((unsigned)v >= (unsigned)n || p >= n || p < -1);
             if (bad) {
                 atomicOr(keys + count + 1, 2ull);
 #ifdef CG_BOUNDS_CHECK
@@ -470,8 +451,6 @@ __global__ void __launch_bounds__(kUnitThreads) peo_unit_kernel(const DenseDesc 
             }
             s_v[lane] = v;
             s_p[lane] = p;
-            const unsigned open = __ballot_sync(0xFFFFFFFFu, p == kParentUnresolved);
-            if (lane == 0) s_open = open;
         }
         // E_b from pos: bit k of word w is set iff pos(32 w + k) < 32 b
         const bool vecpos = ((reinterpret_cast<uintptr_t>(pos_g) & 15) == 0);
@@ -490,48 +469,6 @@ __global__ void __launch_bounds__(kUnitThreads) peo_unit_kernel(const DenseDesc 
                     word |= (__ldg(pos_g + (w << 5) + k) < g0 ? 1u : 0u) << k;
             }
             sE[w] = word;
-        }
-        __syncthreads();
-        // open parents, one vertex per warp
-        unsigned open = s_open;
-        for (int r = 0; open; ++r) {
-            const int j = __ffs(open) - 1;
-            open &= open - 1;
-            if ((r % kUnitWarps) != warp) continue;
-            const int iv = g0 + j;
-            const uint32_t *rv = d.rows + (size_t)s_v[j] * d.words;
-            int best = -1;
-            for (int w0 = 0; w0 < wn; w0 += 32 * kGatherWords) {   // the row words first, then the pos loads
-                uint32_t rw[kGatherWords];
-#pragma unroll
-                for (int k = 0; k < kGatherWords; ++k) {
-                    const int w = w0 + lane + 32 * k;
-                    rw[k] = w < wn ? __ldg(rv + w) : 0u;
-                    if (w == wn - 1) rw[k] &= lastmask;
-                }
-#pragma unroll
-                for (int k = 0; k < kGatherWords; ++k) {
-                    const int w = w0 + lane + 32 * k;
-                    int pu[32];
-#ifdef CG_BOUNDS_CHECK
-                    if (rw[k] && (w << 5) + 31 - __clz(rw[k]) >= n) {
-                        cg_dbg_record(kChkUnitPos, (unsigned long long)((w << 5) + 31 - __clz(rw[k])));
-                        rw[k] = 0u;
-                    }
-#endif
-#pragma unroll
-                    for (int b = 0; b < 32; ++b) pu[b] = (rw[k] >> b) & 1u ? __ldg(pos_g + (w << 5) + b) : -1;
-#pragma unroll
-                    for (int b = 0; b < 32; ++b)
-                        if (pu[b] < iv && pu[b] > best) best = pu[b];
-                }
-            }
-            best = __reduce_max_sync(0xFFFFFFFFu, best);
-            if (lane == 0) {   // also stored for the witness (the last block reads it after the counter)
-                const int pj = best >= 0 ? __ldg(ord_g + best) : -1;
-                s_p[j] = pj;
-                pp_g[iv] = pj;
-            }
         }
         __syncthreads();
         // the check, four positions per warp
@@ -855,9 +792,8 @@ int64_t earlier_mask_words(int n) {
 }
 
 int peo_dense_launch(const DenseDesc *descs, DenseDesc single, int count, const int64_t *voff, int64_t total,
-                     const int32_t *order, const int32_t *pos, int32_t *parent, bool parent_known,
-                     unsigned long long *keys, int num_sms, cudaStream_t stream, uint32_t *emask, int n_max,
-                     bool prefilled, cg_result *res) {
+                     const int32_t *order, const int32_t *pos, int32_t *parent, unsigned long long *keys,
+                     int num_sms, cudaStream_t stream, uint32_t *emask, int n_max, cg_result *res) {
     if (count <= 0) return CG_OK;
     const bool fused = emask && res && total > 0;   // keys initialised by the prep kernel, results by the check
     if (!fused) CG_CUDA_TRY(cudaMemsetAsync(keys, 0xFF, sizeof(unsigned long long) * count, stream));
@@ -868,34 +804,26 @@ int peo_dense_launch(const DenseDesc *descs, DenseDesc single, int count, const 
         const int64_t tiles = ceil_div(wn, 32) * ceil_div(wn, kMaskRows);   // one warp per tile
         const int mask_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(tiles, 8), (int64_t)num_sms * 4));
         const int parent_blocks =
-            parent_known ? 0 : (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n_max, 256), (int64_t)num_sms * 4));
+            (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n_max, 256), (int64_t)num_sms * 4));
         const dim3 grid(mask_blocks + parent_blocks, count);
         unsigned long long *kinit = fused ? keys : nullptr;
-        if (parent_known)
-            peo_prep_kernel<false><<<grid, 256, 0, stream>>>(descs, single, order, pos, parent, emask, mask_blocks,
-                                                             false, kinit);
-        else
-            peo_prep_kernel<true><<<grid, 256, 0, stream>>>(descs, single, order, pos, parent, emask, mask_blocks,
-                                                            prefilled, kinit);
+        peo_prep_kernel<<<grid, 256, 0, stream>>>(descs, single, order, pos, parent, emask, mask_blocks, kinit);
         CG_LAUNCH_CHECK("peo_prep_kernel");
     }
     const int64_t warps_needed = total;
     const int64_t blocks_needed = ceil_div(warps_needed, kPeoThreads / 32);
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(blocks_needed, (int64_t)num_sms * 8));
     cg_result *fres = fused ? res : nullptr;
-    if (parent_known)
-        peo_dense_kernel<true><<<blocks, kPeoThreads, 0, stream>>>(descs, single, count, voff, total, order, pos,
-                                                                   parent, emask, keys, fres);
-    else
-        peo_dense_kernel<false><<<blocks, kPeoThreads, 0, stream>>>(descs, single, count, voff, total, order, pos,
-                                                                    parent, emask, keys, fres);
+    peo_dense_kernel<<<blocks, kPeoThreads, 0, stream>>>(descs, single, count, voff, total, order, pos, parent, emask,
+                                                         keys, fres);
     CG_LAUNCH_CHECK("peo_dense_kernel");
     if (res && !fused) return finalize_launch(descs, single, count, keys, order, parent, res, stream);
     return CG_OK;
 }
 
 int peo_unit_launch(const DenseDesc *descs, DenseDesc single, int count, int n_max, bool vec, const int32_t *order,
-                    const int32_t *pos, int32_t *ppos, unsigned long long *keys, cg_result *res, cudaStream_t stream) {
+                    const int32_t *pos, const int32_t *ppos, unsigned long long *keys, cg_result *res,
+                    cudaStream_t stream) {
     if (count <= 0 || n_max <= 0) return set_error(CG_EINVAL, "position-ordered check needs vertices");
     if (count > 65535) return set_error(CG_EINVAL, "too many graphs for one check launch (%d)", count);
     const dim3 grid((unsigned)ceil_div(n_max, 32), (unsigned)count);
