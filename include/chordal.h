@@ -186,11 +186,11 @@ int cg_chordal_test_mcs_dense(cg_context *ctx, const cg_dense *g, cg_result *res
                               cudaStream_t stream);
 
 /*
- * LexBFS order of a CSR graph (Section 4.2 in its O(N + M) form: each class a
- * list sorted by id, only the pivot's neighbours move).  One CTA walks the n
- * steps (warp 0; all its warps for rows longer than 32 neighbours) with the
- * partition state in the context workspace: 60 n bytes plus 8 bytes per
- * sort key slot (the next power of two >= n), 68-76 B per vertex.
+ * LexBFS order of a CSR graph (Section 4.2 in its O(N + M) form: only the
+ * pivot's neighbours move).  One CTA numbers up to 32 vertices per pass over
+ * the rows of the next ones, each class a segment of a vertex arena in id
+ * order, with the partition state in the context workspace: 60 n bytes plus 8
+ * bytes per sort key slot (the next power of two >= n), 68-76 B per vertex.
  *   g      device CSR graph (sorted, symmetric, no loops; checked only when
  *          cfg.validate, which then synchronises the stream)
  *   order  device int32[n] (written);  pos  device int32[n] (written) or NULL

@@ -156,6 +156,9 @@ int fused_dense_plan(int n_max, int threads, FusedPlan *plan) {
         return set_error(CG_EINVAL, "fused batch path supports n <= %d (got %d)", kFusedMaxN, n_max);
     const int n = std::max(n_max, 1);
     FusedPlan p{};
+    // for batches that fill the GPU: with 64 / 128 / 256 / 512 threads 1,200 graphs of 250 vertices take 140 / 170 /
+    // 217 / 546 us, of 1,000 723 / 791 / 841 / 1,971, of 2,000 2,883 / 2,011 / 2,043 / 4,045.  (Two graphs of 250 take
+    // 106 / 83 / 70 / 87, of 1,000 471 / 307 / 236 / 244: cg_batch_autotune finds that.)
     if (threads == 0) threads = n <= 256 ? 64 : n <= 2048 ? 128 : 256;
     if (threads != 64 && threads != 128 && threads != 256 && threads != 512)
         return set_error(CG_EINVAL, "fused batch path: unsupported CTA size %d", threads);

@@ -391,7 +391,7 @@ int run_single_dense(cg_context *ctx, const cg_dense *g, int32_t *order_out, int
                                 res);
     }
     // with a result wanted, the search also records the parents of its pivots
-    // by position (one store per step) and initialises the check's keys
+    // by position and initialises the check's keys
     const bool stage = res && peo_stage_ok(d);
     uint32_t *emask = stage ? at<uint32_t>(ctx, base + sc.o_emask) : nullptr;
     {

@@ -130,7 +130,7 @@ int sweep_order_launch(const DenseDesc &d, const LexPlan &plan, void *gstate, in
 size_t mcs_workspace_bytes(int n);   // 16-byte aligned
 int mcs_dense_launch(DenseDesc d, int32_t *order, int32_t *pos, void *ws, cudaStream_t stream);
 
-// ---- CSR LexBFS (lexbfs_csr.cu): one CTA per graph (warp 0 walks the steps), state in `ws`
+// ---- CSR LexBFS (lexbfs_csr.cu): one CTA per graph, panels of up to 32 pivots, state in `ws`
 size_t lexbfs_csr_workspace_bytes(int64_t n, int64_t max_deg);
 int lexbfs_csr_launch(int n, int64_t max_deg, const int64_t *row_ptr, const int32_t *col, int64_t nnz, int32_t *order,
                       int32_t *pos, int32_t *parent, void *ws, int num_sms, cudaStream_t stream);

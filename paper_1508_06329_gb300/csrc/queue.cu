@@ -219,7 +219,7 @@ int launch_batch(cg_queue *q, Slot &s, bool dry = false, size_t *bytes_out = nul
         return set_error(CG_EINVAL, "batch larger than the slot's staging");
     }
 csr_part:
-    // sparse CSR requests: one warp each on the slot stream
+    // sparse CSR requests: one CTA each on the slot stream
     for (int i = 0; i < count; ++i) {
         const Request &r = s.reqs[i];
         if (r.route != kRouteCsr) continue;
