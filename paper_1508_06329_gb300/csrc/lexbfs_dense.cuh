@@ -1361,24 +1361,6 @@ __device__ __forceinline__ int panel_windows(const uint32_t *__restrict__ rows, 
     return i;
 }
 
-// The vertices from position i on, after windows that did not pay: a panel of
-// steps, then windows as long as they pay, four panels of steps, and so on.
-template <int STATE, int T>
-__device__ __forceinline__ void panel_rest(const uint32_t *__restrict__ rows, int stride, int n, int i, int cap,
-                                           unsigned char *gstate, int32_t *__restrict__ order,
-                                           int32_t *__restrict__ pos, int32_t *ppos_out, uint32_t *emask) {
-    int span = 1;
-#pragma unroll 1
-    while (i < n) {
-        const int i0 = i;
-        i = panel_narrow<STATE, T>(rows, stride, n, i, cap, gstate, order, pos, ppos_out, emask, span);
-        span = min(4 * span, kStepsMost);
-        // the next window that does not pay is the last one, unless the steps did not pay either
-        int lost = i - i0 < kStepsBelow ? 0 : panel_lost_limit(n);
-        i = panel_windows<STATE, T>(rows, stride, n, i, cap, gstate, order, pos, ppos_out, emask, lost, span);
-    }
-}
-
 // One CTA computes the LexBFS order of one graph (rows: n rows of `stride`
 // words in global memory; gstate: this CTA's workspace).  order gets the vertices
 // by position; pos (nullable) its inverse; ppos (nullable) p(order[i]) by position
@@ -1407,9 +1389,18 @@ __device__ __forceinline__ void lexbfs_panels(const uint32_t *__restrict__ rows,
         if (t == 0 && ppos_out) cg_arr(ppos_out, n, kChkPpos)[0] = -1;
         __syncthreads();
     }
+    // windows as long as they pay, then a panel of steps, windows again, four panels of steps, and so on
     int lost = 0, span = 1;
-    const int i = panel_windows<STATE, T>(rows, stride, n, 0, cap, gstate, order, pos, ppos_out, emask, lost, span);
-    if (i < n) panel_rest<STATE, T>(rows, stride, n, i, cap, gstate, order, pos, ppos_out, emask);
+#pragma unroll 1
+    for (int i = 0;;) {
+        i = panel_windows<STATE, T>(rows, stride, n, i, cap, gstate, order, pos, ppos_out, emask, lost, span);
+        if (i >= n) return;
+        const int i0 = i;
+        i = panel_narrow<STATE, T>(rows, stride, n, i, cap, gstate, order, pos, ppos_out, emask, span);
+        span = min(4 * span, kStepsMost);
+        // the next window that does not pay is the last one, unless the steps did not pay either
+        lost = i - i0 < kStepsBelow ? 0 : panel_lost_limit(n);
+    }
 }
 
 }  // namespace cg
