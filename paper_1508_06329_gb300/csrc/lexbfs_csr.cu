@@ -852,7 +852,7 @@ __device__ void csr_steps(const CsrState &s, CsrShared *sh, const CsrGraph &g, i
                 adj |= is;
                 if (__ballot_sync(kFull, is) && lane == k) known = true;
             }
-            const bool fresh = !known && cw != kNumberedCls;
+            const bool fresh = !known && cw != kNumberedCls && w != x;
             const uint32_t met = __ballot_sync(kFull, fresh), room = __ballot_sync(kFull, y < 0 || y == x);
             if (__popc(met) > __popc(room)) {
                 stop = true;
